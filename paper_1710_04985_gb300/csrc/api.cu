@@ -57,29 +57,43 @@ struct Levels {
     int* count0 = nullptr;
     int* count = nullptr;
     int method = SPTRSV_ANALYSIS_SWEEP;  // the analysis that produced these levels
-    // Part-ordered copy (SPTRSV_ALGO_SELF_PARTITIONED, built on first use and
-    // again when the part size changes): position k holds row qord[k], rows
-    // in parts of qS consecutive rows, by level inside a part; columns
-    // renumbered to positions (qipos); xq is the publication buffer of its
-    // solves (position order).
+    // Part order (SPTRSV_ALGO_SELF_PARTITIONED, built on first use and again
+    // when the part size changes): position k holds row qord[k], rows in parts
+    // of qS consecutive rows, by level inside a part; qipos is its inverse and
+    // xq the publication buffer of its solves (position order).
     // qpart: first position of each part (qnparts + 1 entries, parts in the
-    // order they are handed out), qmaxpart the longest part, qnblocks the
-    // independent blocks the substitution order splits into.
+    // order they are handed out), qrow the lowest row of each part, qmaxpart
+    // the longest part, qnblocks the independent blocks the substitution order
+    // splits into.
     int qS = 0;
     int* qord = nullptr;
     int* qipos = nullptr;
-    int* qptr = nullptr;
-    int* qidx = nullptr;
-    void* qvals = nullptr;
     void* xq = nullptr;
     int* qpart = nullptr;
+    int* qrow = nullptr;
     int qnparts = 0, qmaxpart = 0, qnblocks = 0;
-    // FP32 values and publication buffers of the level- and part-ordered
+    // Sliced copy of the matrix in part order, per log2(lanes) (built on first
+    // use; layout in solve_parts.cu).  wide: its padding would take more than
+    // kMaxPadding times the stored entries, so it is not built and solves of
+    // this width run on the level-ordered copy.
+    struct Slices {
+        bool built = false, wide = false;
+        int ngroups = 0;
+        long long slots = 0;
+        int4* grp = nullptr;
+        int* grp_ptr = nullptr;
+        int* cols = nullptr;
+        void* vals = nullptr;
+        void* dinv = nullptr;
+        // FP32 values, for the FP32 solves of a refined F64 plan
+        void* vals32 = nullptr;
+        void* dinv32 = nullptr;
+    } qs[6];
+    // FP32 values of the level-ordered copy and FP32 publication buffers of both
     // copies of an F64 plan, for the FP32 solves of the refined solve (built
     // on first use from the plan's FP32 copy of the values).
     void* pvals32 = nullptr;
     void* xp32 = nullptr;
-    void* qvals32 = nullptr;
     void* xq32 = nullptr;
     // multi-RHS solves on the level-ordered copy: publication buffer
     // [n][nrhs] in position order (grown on demand)
@@ -87,18 +101,32 @@ struct Levels {
     size_t xpm_bytes = 0;
 };
 
+// Sliced copies larger than this many times the stored entries are not built.
+// Each slot costs a load in the solve; a width at which eight in nine slots are
+// empty is never the one to use.
+constexpr long long kMaxPadding = 8;
+
+void free_slices(Levels::Slices& q) {
+    cudaFree(q.grp);
+    cudaFree(q.grp_ptr);
+    cudaFree(q.cols);
+    cudaFree(q.vals);
+    cudaFree(q.dinv);
+    cudaFree(q.vals32);
+    cudaFree(q.dinv32);
+    q = Levels::Slices();
+}
+
 void free_parts(Levels& L) {
     cudaFree(L.qord);
     cudaFree(L.qipos);
-    cudaFree(L.qptr);
-    cudaFree(L.qidx);
-    cudaFree(L.qvals);
     cudaFree(L.xq);
     cudaFree(L.qpart);
-    cudaFree(L.qvals32);
+    cudaFree(L.qrow);
     cudaFree(L.xq32);
-    L.qord = L.qipos = L.qptr = L.qidx = L.qpart = nullptr;
-    L.qvals = L.xq = L.qvals32 = L.xq32 = nullptr;
+    for (Levels::Slices& q : L.qs) free_slices(q);
+    L.qord = L.qipos = L.qpart = L.qrow = nullptr;
+    L.xq = L.xq32 = nullptr;
     L.qS = L.qnparts = L.qmaxpart = L.qnblocks = 0;
 }
 
@@ -685,7 +713,28 @@ sptrsv_status_t build_column(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     return SPTRSV_OK;
 }
 
-// Re-gathers the values of every level-ordered copy from the plan's values.
+// Pattern and part order of one direction, for the slicing kernels.
+SliceParams slice_params(sptrsv_plan_t P, bool trans, const Levels::Slices& q) {
+    const Levels& L = trans ? P->trn : P->fwd;
+    SliceParams p;
+    p.n = P->n;
+    p.ptr = trans ? P->tptr : P->rowptr;
+    p.idx = trans ? P->tidx : P->colidx;
+    p.vmap = trans ? P->tmap : nullptr;
+    p.upper = (trans ? !P->upper : P->upper) ? 1 : 0;
+    p.qord = L.qord;
+    p.qipos = L.qipos;
+    p.part_ptr = L.qpart;
+    p.part_row = L.qrow;
+    p.nparts = L.qnparts;
+    p.max_part = L.qmaxpart;
+    p.grp_ptr = q.grp_ptr;
+    p.ngroups = q.ngroups;
+    p.status = P->status;
+    return p;
+}
+
+// Re-gathers the values of every copy from the plan's values.
 cudaError_t refresh_permuted(sptrsv_plan_t P, cudaStream_t s) {
     for (int d = 0; d < 2; ++d) {
         Levels& L = d ? P->trn : P->fwd;
@@ -699,33 +748,32 @@ cudaError_t refresh_permuted(sptrsv_plan_t P, cudaStream_t s) {
     }
     for (int d = 0; d < 2; ++d) {
         Levels& L = d ? P->trn : P->fwd;
-        if (!L.qvals) continue;
-        cudaError_t e = launch_permute_rows(P->f64, P->n, d ? P->tptr : P->rowptr,
-                                            d ? P->tidx : P->colidx, d ? P->tmap : nullptr,
-                                            P->vals, L.qord, L.qipos, L.qptr, nullptr, L.qvals,
-                                            P->num_sms * 16, s, copy_diag(P, d),
-                                            d ? !P->upper : P->upper);
-        if (e != cudaSuccess) return e;
-    }
-    // the FP32 copies of the refined solve, from the refreshed FP32 values
-    for (int d = 0; d < 2 && P->vals32; ++d) {
-        Levels& L = d ? P->trn : P->fwd;
-        for (int parts = 0; parts < 2; ++parts) {
-            void* v = parts ? L.qvals32 : L.pvals32;
-            if (!v) continue;
-            cudaError_t e = launch_permute_rows(
-                false, P->n, d ? P->tptr : P->rowptr, d ? P->tidx : P->colidx,
-                d ? P->tmap : nullptr, P->vals32, parts ? L.qord : L.jlev,
-                parts ? L.qipos : L.ipos, parts ? L.qptr : L.pptr, nullptr, v, P->num_sms * 16, s,
-                copy_diag(P, d), d ? !P->upper : P->upper);
+        for (int w = 0; w < 6; ++w) {
+            Levels::Slices& q = L.qs[w];
+            if (!q.vals) continue;
+            cudaError_t e = launch_fill_slices(P->f64, slice_params(P, d, q), 1 << w, q.grp,
+                                               P->vals, nullptr, q.vals, q.dinv, s);
+            if (e == cudaSuccess && q.vals32 && P->vals32)
+                e = launch_fill_slices(false, slice_params(P, d, q), 1 << w, q.grp, P->vals32,
+                                       nullptr, q.vals32, q.dinv32, s);
             if (e != cudaSuccess) return e;
         }
+    }
+    // the level-ordered FP32 copies of the refined solve, from the refreshed FP32 values
+    for (int d = 0; d < 2 && P->vals32; ++d) {
+        Levels& L = d ? P->trn : P->fwd;
+        if (!L.pvals32) continue;
+        cudaError_t e = launch_permute_rows(
+            false, P->n, d ? P->tptr : P->rowptr, d ? P->tidx : P->colidx,
+            d ? P->tmap : nullptr, P->vals32, L.jlev, L.ipos, L.pptr, nullptr, L.pvals32,
+            P->num_sms * 16, s, copy_diag(P, d), d ? !P->upper : P->upper);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-// Largest part whose unknowns fit a block's shared memory (the blocked
-// kernel keeps a tile's unknowns there).
+// Largest part whose unknowns fit a block's shared memory (the partitioned
+// kernel keeps them there).
 int max_part_rows(sptrsv_plan_t P) {
     const int esize = P->f64 ? 8 : 4;
     const int room = P->smem_optin - 128;
@@ -743,14 +791,12 @@ int resolve_part_rows(sptrsv_plan_t P) {
     return (int)S;
 }
 
-// Part-ordered copy of one direction's pattern and values for the
-// partitioned solve (layout in solve_parts.cu): the independent blocks of the
-// substitution order and their depths, the parts (balanced pieces of long
-// blocks, short blocks packed together) and their hand-out order (deepest
-// block first), the level order jlev stably re-sorted by part, its inverse,
-// the copy with columns renumbered to positions, its self-check (every entry
-// names its own or an earlier position) and the publication buffer.
-// Allocates and synchronises s.
+// Part order of one direction for the partitioned solve (solve_parts.cu): the
+// independent blocks of the substitution order and their depths, the parts
+// (balanced pieces of long blocks, short blocks packed together) and their
+// hand-out order (deepest block first), the level order jlev stably re-sorted
+// by part, its inverse and the publication buffer.  Allocates and synchronises
+// s.
 sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     Levels& L = trans ? P->trn : P->fwd;
     const int S = resolve_part_rows(P);
@@ -758,28 +804,23 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     CK(cudaStreamSynchronize(s));
     free_parts(L);
-    const int n = P->n, nnz = P->nnz;
+    const int n = P->n;
     const bool upper = trans ? !P->upper : P->upper;
     const size_t esize = P->f64 ? sizeof(double) : sizeof(float);
     const int* ptr = trans ? P->tptr : P->rowptr;
     const int* idx = trans ? P->tidx : P->colidx;
-    const int* vmap = trans ? P->tmap : nullptr;
-    const size_t nz = nnz > 0 ? (size_t)nnz : 1;
     const size_t N = (size_t)n;
     const int hist_n = radix_hist_entries(n);
-    int *qord = nullptr, *qipos = nullptr, *qptr = nullptr, *qidx = nullptr, *scratch = nullptr;
-    int* qpart = nullptr;
-    void *qvals = nullptr, *xq = nullptr;
+    int *qord = nullptr, *qipos = nullptr, *scratch = nullptr;
+    int *qpart = nullptr, *qrow = nullptr;
+    void* xq = nullptr;
     cudaError_t e = cudaMalloc(&qord, sizeof(int) * N);
     if (e == cudaSuccess) e = cudaMalloc(&qipos, sizeof(int) * N);
-    if (e == cudaSuccess) e = cudaMalloc(&qptr, sizeof(int) * (N + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&qidx, sizeof(int) * nz);
-    if (e == cudaSuccess) e = cudaMalloc(&qvals, esize * nz);
     if (e == cudaSuccess) e = cudaMalloc(&xq, esize * N);
     // scratch (ints): diff n+1, cover n+2, bflag n, bscan n+1, bstart n+1,
     // depth n, pflag n, pscan n+1, pstart n+1, pkey n, horder n, prank n,
-    // psize n, rowkey n, lens n, 2 counters | radix sort: 4 n + 2 hist
-    const size_t scratch_ints = 22 * N + 16 + 2 * (size_t)hist_n;
+    // psize n, rowkey n, 8 counters | radix sort: 4 n + 2 hist
+    const size_t scratch_ints = 21 * N + 16 + 2 * (size_t)hist_n;
     if (e == cudaSuccess) e = cudaMalloc(&scratch, sizeof(int) * scratch_ints);
     int* diff = scratch;
     int* cover = diff + (N + 1);
@@ -795,8 +836,7 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     int* prank = horder + N;
     int* psize = prank + N;
     int* rowkey = psize + N;
-    int* lens = rowkey + N;
-    int* counters = lens + N;  // [0] longest part
+    int* counters = rowkey + N;  // [0] longest part
     int* k_a = counters + 8;
     int* v_a = k_a + N;
     int* k_b = v_a + N;
@@ -826,6 +866,7 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && (np < 1 || np > n || nb < 1 || nb > n)) e = cudaErrorUnknown;
     if (e == cudaSuccess) e = cudaMalloc(&qpart, sizeof(int) * ((size_t)np + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&qrow, sizeof(int) * (size_t)np);
     // hand-out order: latest start first -- by the block's slack (deepest
     // level minus its depth) plus the piece's share of the block's levels,
     // then order of substitution.  SPTRSV_PART_ORDER=2: by piece index (every
@@ -858,20 +899,15 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
                                   v_b, hist, hist_scan, P->status, s);
     }
     if (e == cudaSuccess) e = launch_inverse_perm(horder, np, prank, s);
-    if (e == cudaSuccess) e = launch_part_sizes(np, horder, pstart, psize, counters, s);
+    if (e == cudaSuccess) e = launch_part_sizes(n, np, upper, horder, pstart, psize, qrow, counters,
+                                               s);
     if (e == cudaSuccess) e = launch_exclusive_scan(psize, qpart, np, s);
     if (e == cudaSuccess) e = launch_row_part_keys(n, L.jlev, upper, pscan, prank, rowkey, s);
-    // the copy: rows by part (hand-out order), by level inside a part
+    // rows by part (hand-out order), by level inside a part
     if (e == cudaSuccess)
         e = radix_sort_values(rowkey, L.jlev, n, bits_for(np - 1), qord, k_a, v_a, k_b, v_b,
                               hist, hist_scan, P->status, s);
     if (e == cudaSuccess) e = launch_inverse_perm(qord, n, qipos, s);
-    if (e == cudaSuccess) e = launch_ordered_lengths(n, ptr, qord, lens, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(lens, qptr, n, s);
-    if (e == cudaSuccess)
-        e = launch_permute_rows(P->f64, n, ptr, idx, vmap, P->vals, qord, qipos, qptr, qidx,
-                                qvals, P->num_sms * 16, s, copy_diag(P, trans), upper);
-    if (e == cudaSuccess) e = launch_verify_permuted(n, qptr, qidx, P->status, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&maxpart, counters, sizeof(int),
                                               cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -884,35 +920,101 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     if (rc != SPTRSV_OK) {
         cudaFree(qord);
         cudaFree(qipos);
-        cudaFree(qptr);
-        cudaFree(qidx);
-        cudaFree(qvals);
         cudaFree(xq);
         cudaFree(qpart);
+        cudaFree(qrow);
         return rc;
     }
     L.qS = S;
     L.qord = qord;
     L.qipos = qipos;
-    L.qptr = qptr;
-    L.qidx = qidx;
-    L.qvals = qvals;
     L.xq = xq;
     L.qpart = qpart;
+    L.qrow = qrow;
     L.qnparts = np;
     L.qmaxpart = maxpart;
     L.qnblocks = nb;
     return SPTRSV_OK;
 }
 
-// FP32 values (gathered from the plan's FP32 copy vals32) and an FP32
-// publication buffer for the level-ordered (parts = false) or part-ordered
-// (parts = true) copy of an F64 plan, whose pattern must exist.  Allocates.
-sptrsv_status_t build_copy_f32(sptrsv_plan_t P, bool trans, bool parts, cudaStream_t s) {
+// Sliced copy of one direction's matrix in part order (which must exist) for
+// one sub-warp width: the row groups (runs of equal level inside a part, cut
+// into groups of at most 32/lanes rows), their shapes, columns and values,
+// with the self-check of the fill kernel (every entry names an earlier
+// position outside its group).  Allocates and synchronises s.
+sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_t s) {
     Levels& L = trans ? P->trn : P->fwd;
-    void*& vals = parts ? L.qvals32 : L.pvals32;
-    void*& xpub = parts ? L.xq32 : L.xp32;
-    if (vals) return SPTRSV_OK;
+    const int w = log2_lanes(lanes);
+    if (L.qs[w].built) return SPTRSV_OK;
+    if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
+    const int n = P->n;
+    const size_t N = (size_t)n;
+    const size_t esize = P->f64 ? sizeof(double) : sizeof(float);
+    Levels::Slices q;
+    int* scratch = nullptr;
+    int h[2] = {0, 0};  // groups, slices
+    cudaError_t e = cudaMalloc(&scratch, sizeof(int) * (5 * N + 5));
+    int* flag = scratch;           // of the runs; then the group starts
+    int* scan = flag + (N + 1);    // of the run flags, then of the group flags
+    int* rstart = scan + (N + 1);  // run starts; then the groups' slice counts
+    int* gflag = rstart + (N + 1);
+    int* base = gflag + N;
+    if (e == cudaSuccess) e = cudaMalloc(&q.grp_ptr, sizeof(int) * ((size_t)L.qnparts + 1));
+    if (e == cudaSuccess) e = launch_run_flags(n, L.qord, L.lev, flag, s);
+    if (e == cudaSuccess) e = launch_part_flag_starts(L.qnparts, L.qpart, flag, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(flag, scan, n, s);
+    if (e == cudaSuccess) e = launch_flag_scatter(n, flag, scan, rstart, s);
+    if (e == cudaSuccess) e = launch_group_flags(n, 32 / lanes, scan, rstart, gflag, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(gflag, scan, n, s);
+    if (e == cudaSuccess) e = launch_part_groups(L.qnparts, L.qpart, scan, q.grp_ptr, s);
+    if (e == cudaSuccess) e = launch_flag_scatter(n, gflag, scan, flag, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&h[0], scan + n, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && (h[0] < L.qnparts || h[0] > n)) e = cudaErrorUnknown;
+    q.ngroups = h[0];
+    const int *gstart = flag, *cnt = rstart;
+    if (e == cudaSuccess) e = cudaMalloc(&q.grp, sizeof(int4) * (size_t)q.ngroups);
+    const SliceParams sp = slice_params(P, trans, q);
+    if (e == cudaSuccess) e = launch_group_shapes(sp, lanes, gstart, q.grp, rstart, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(cnt, base, q.ngroups, s);
+    if (e == cudaSuccess) e = launch_group_bases(q.ngroups, base, q.grp, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&h[1], base + q.ngroups, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    // a lane holds at most its rows' entries, so the slices are at most nnz
+    if (e == cudaSuccess && (h[1] < 0 || h[1] > P->nnz)) e = cudaErrorUnknown;
+    q.slots = 32ll * h[1];
+    q.wide = q.slots > kMaxPadding * P->nnz + (1 << 20);
+    const size_t slots = q.slots > 0 ? (size_t)q.slots : 1;
+    if (e == cudaSuccess && !q.wide) {
+        e = cudaMalloc(&q.cols, sizeof(int) * slots);
+        if (e == cudaSuccess) e = cudaMalloc(&q.vals, esize * slots);
+        if (e == cudaSuccess && !P->unit) e = cudaMalloc(&q.dinv, esize * N);
+        if (e == cudaSuccess)
+            e = launch_fill_slices(P->f64, sp, lanes, q.grp, P->vals, q.cols, q.vals, q.dinv, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    sptrsv_status_t rc = e == cudaSuccess ? SPTRSV_OK
+                         : e == cudaErrorUnknown ? SPTRSV_ERR_INTERNAL : cuda_fail(e);
+    int row = -1;
+    if (rc == SPTRSV_OK && take_status(P, s, &row) != SPTRSV_OK) rc = SPTRSV_ERR_INTERNAL;
+    cudaFree(scratch);
+    if (rc != SPTRSV_OK) {
+        free_slices(q);
+        return rc;
+    }
+    q.built = true;
+    L.qs[w] = q;
+    return SPTRSV_OK;
+}
+
+// FP32 values (gathered from the plan's FP32 copy vals32) and an FP32
+// publication buffer for the level-ordered copy of an F64 plan, whose pattern
+// must exist.  Allocates.
+sptrsv_status_t build_copy_f32(sptrsv_plan_t P, bool trans, cudaStream_t s) {
+    Levels& L = trans ? P->trn : P->fwd;
+    if (L.pvals32) return SPTRSV_OK;
     if (!P->vals32 && P->nnz > 0) return SPTRSV_ERR_NOT_SUPPORTED;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     const size_t nz = P->nnz > 0 ? (size_t)P->nnz : 1;
@@ -922,16 +1024,39 @@ sptrsv_status_t build_copy_f32(sptrsv_plan_t P, bool trans, bool parts, cudaStre
     if (e == cudaSuccess)
         e = launch_permute_rows(false, P->n, trans ? P->tptr : P->rowptr,
                                 trans ? P->tidx : P->colidx, trans ? P->tmap : nullptr, P->vals32,
-                                parts ? L.qord : L.jlev, parts ? L.qipos : L.ipos,
-                                parts ? L.qptr : L.pptr, nullptr, v, P->num_sms * 16, s,
+                                L.jlev, L.ipos, L.pptr, nullptr, v, P->num_sms * 16, s,
                                 copy_diag(P, trans), trans ? !P->upper : P->upper);
     if (e != cudaSuccess) {
         cudaFree(v);
         cudaFree(xq);
         return cuda_fail(e);
     }
-    vals = v;
-    xpub = xq;
+    L.pvals32 = v;
+    L.xp32 = xq;
+    return SPTRSV_OK;
+}
+
+// The same for the sliced copy of one width.
+sptrsv_status_t build_slices_f32(sptrsv_plan_t P, bool trans, int lanes, cudaStream_t s) {
+    Levels& L = trans ? P->trn : P->fwd;
+    Levels::Slices& q = L.qs[log2_lanes(lanes)];
+    if (q.vals32 && L.xq32) return SPTRSV_OK;
+    if (!P->vals32 && P->nnz > 0) return SPTRSV_ERR_NOT_SUPPORTED;
+    if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
+    if (!L.xq32) CK(cudaMalloc(&L.xq32, sizeof(float) * (size_t)P->n));
+    void *v = nullptr, *di = nullptr;
+    cudaError_t e = cudaMalloc(&v, sizeof(float) * (q.slots > 0 ? (size_t)q.slots : 1));
+    if (e == cudaSuccess && !P->unit) e = cudaMalloc(&di, sizeof(float) * (size_t)P->n);
+    if (e == cudaSuccess)
+        e = launch_fill_slices(false, slice_params(P, trans, q), lanes, q.grp, P->vals32, nullptr,
+                               v, di, s);
+    if (e != cudaSuccess) {
+        cudaFree(v);
+        cudaFree(di);
+        return cuda_fail(e);
+    }
+    q.vals32 = v;
+    q.dinv32 = di;
     return SPTRSV_OK;
 }
 
@@ -982,6 +1107,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
                           cudaStream_t s, double* xacc = nullptr, long long ldacc = 0,
                           bool acc_first = false) {
     const bool mrhs = nrhs > 1;
+    const bool f32_of_f64 = !f64 && P->f64;
     // multi-RHS solves have a launch shape of their own (sptrsv_set_mrhs_tuning);
     // a single-RHS solve takes its algorithm's shape if one was set
     const int a = (int)algo;
@@ -995,17 +1121,23 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     if (algo == SPTRSV_ALGO_SELF_CHAINS && !mrhs) ST(build_chain(P, trans, lanes, s));
     // The copies hold the plan's element type, and FP32 values beside them
     // for the FP32 solves of a refined F64 plan (f64 != P->f64).
-    const bool f32_of_f64 = !f64 && P->f64;
     if (f64 != P->f64 && !f32_of_f64) return SPTRSV_ERR_INVALID_ARG;
+    bool parts = algo == SPTRSV_ALGO_SELF_PARTITIONED && !mrhs;
+    if (parts) {
+        ST(build_parts(P, trans, s));
+        ST(build_slices(P, trans, lanes, s));
+        parts = !(trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].wide;
+        if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
+    }
     const bool blocked = algo == SPTRSV_ALGO_SELF_BLOCKED && !mrhs;
-    const bool permuted = (algo == SPTRSV_ALGO_SELF_PERMUTED || blocked) && !mrhs;
+    // a partitioned solve whose sliced copy would be mostly padding runs on the
+    // level-ordered copy (bitwise the same result)
+    const bool permuted = (algo == SPTRSV_ALGO_SELF_PERMUTED || blocked ||
+                           (algo == SPTRSV_ALGO_SELF_PARTITIONED && !parts)) && !mrhs;
     if (permuted) ST(build_permuted(P, trans, s));
-    if (permuted && f32_of_f64) ST(build_copy_f32(P, trans, false, s));
+    if (permuted && f32_of_f64) ST(build_copy_f32(P, trans, s));
     const bool column = algo == SPTRSV_ALGO_SELF_COLUMN && !mrhs;
     if (column) ST(build_column(P, trans, s));
-    const bool parts = algo == SPTRSV_ALGO_SELF_PARTITIONED && !mrhs;
-    if (parts) ST(build_parts(P, trans, s));
-    if (parts && f32_of_f64) ST(build_copy_f32(P, trans, true, s));
     // multi-RHS solves of the copying forms run on the level-ordered copy
     // (the shared-memory tiles of the blocked and partitioned forms hold one
     // column): the multi-RHS kernel with a position-ordered publication buffer
@@ -1015,7 +1147,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     if (mrhs_copy) {
         Levels& Lw = trans ? P->trn : P->fwd;
         ST(build_permuted(P, trans, s));
-        if (f32_of_f64) ST(build_copy_f32(P, trans, false, s));
+        if (f32_of_f64) ST(build_copy_f32(P, trans, s));
         ST(ensure_bytes(&Lw.xpm, &Lw.xpm_bytes,
                         (f64 ? sizeof(double) : sizeof(float)) * (size_t)P->n * nrhs, s));
     }
@@ -1080,31 +1212,36 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         ST(prof_end(P, s));
         launches = 2;
     } else if (parts) {
-        // The blocked kernel on the part-ordered copy, one part per tile.
-        // Rows publish to L.xq and store x(i) for the caller; b(i) is read
-        // once, by row i, before x(i) is written, so in place needs no copy.
-        p.ptr = L.qptr;
-        p.idx = L.qidx;
+        // On the sliced copy, one part per thread block.  Rows publish to L.xq
+        // and store x(i) for the caller; b(i) is read by row i before x(i) is
+        // written, so in place needs no copy.
+        const Levels::Slices& q = L.qs[log2_lanes(lanes)];
+        p.ptr = nullptr;
+        p.idx = q.cols;
         p.vmap = nullptr;
-        p.vals = f32_of_f64 ? L.qvals32 : L.qvals;
+        p.vals = f32_of_f64 ? q.vals32 : q.vals;
+        p.dinv = f32_of_f64 ? q.dinv32 : q.dinv;
         p.xp = f32_of_f64 ? L.xq32 : L.xq;
         p.prescaled = P->unit ? 0 : 1;
         p.jlev = L.qord;
-        p.diag_first = 0;  // the copy stores an upper row's entries in descending order
         p.part_ptr = L.qpart;
+        p.part_row = L.qrow;
         p.nparts = L.qnparts;
+        p.max_part = L.qmaxpart;
+        p.grp = q.grp;
+        p.grp_ptr = q.grp_ptr;
         CK(launch_prep_self(f64, P->n, 1, p.xp, 1, nullptr, 0, nullptr, P->counters,
                             P->num_sms * 8, s));
         const int cl = P->part_cluster;
         const long long groups = ((long long)L.qnparts + cl - 1) / cl;
-        long long grid = blocked_resident_blocks(f64, lanes, cl, block, L.qmaxpart, P->num_sms);
+        long long grid = part_resident_blocks(f64, lanes, cl, block, L.qmaxpart, P->num_sms);
         if (grid < cl) return SPTRSV_ERR_INVALID_ARG;  // this shape cannot run
         if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
         if (grid > groups * cl) grid = groups * cl;
         grid = grid / cl * cl;
         if (grid < cl) grid = cl;
         ST(prof_begin(P, s));
-        CK(launch_blocked_k1(f64, lanes, p, L.qmaxpart, (int)grid, block, s, cl));
+        CK(launch_part_k1(f64, lanes, p, (int)grid, block, cl, s));
         ST(prof_end(P, s));
         launches = 2;
     } else if (mrhs_copy) {
@@ -1149,8 +1286,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
         if (blocked) {
             const long long tiles = ((long long)P->n + P->tile_rows - 1) / P->tile_rows;
-            long long grid = blocked_resident_blocks(f64, lanes, 1, block, P->tile_rows,
-                                                     P->num_sms);
+            long long grid = blocked_resident_blocks(f64, lanes, block, P->tile_rows, P->num_sms);
             if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
             if (grid > tiles) grid = tiles;
             if (grid < 1) grid = 1;
@@ -1420,7 +1556,12 @@ sptrsv_status_t sptrsv_prepare(sptrsv_plan_t plan, int transpose, sptrsv_algo_t 
         case SPTRSV_ALGO_SELF_CHAINS: ST(build_chain(P, trans, lanes, s)); break;
         case SPTRSV_ALGO_SELF_PERMUTED:
         case SPTRSV_ALGO_SELF_BLOCKED: ST(build_permuted(P, trans, s)); break;
-        case SPTRSV_ALGO_SELF_PARTITIONED: ST(build_parts(P, trans, s)); break;
+        case SPTRSV_ALGO_SELF_PARTITIONED:
+            ST(build_parts(P, trans, s));
+            ST(build_slices(P, trans, lanes, s));
+            if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].wide)
+                ST(build_permuted(P, trans, s));
+            break;
         case SPTRSV_ALGO_SELF_COLUMN: ST(build_column(P, trans, s)); break;
         default: break;
     }
@@ -1484,7 +1625,7 @@ sptrsv_status_t refine_in_passes(sptrsv_plan_t P, const double* d_b, double* d_x
     const int n = P->n;
     const int grid16 = P->num_sms * 16;
     ST(build_permuted(P, false, s));
-    ST(build_copy_f32(P, false, false, s));
+    ST(build_copy_f32(P, false, s));
     const Levels& L = P->fwd;
     const int S = kRefineMaxSteps + 1;
     const size_t want = (size_t)S * n;

@@ -33,9 +33,15 @@ struct SolveParams {
     int kbeg, cnt;        // level-scheduled: this launch's slice of jlev
     void* xp;             // level-ordered solve: publication buffer in position
                           // order (nullptr: rows publish to x itself)
-    const int* part_ptr;  // blocked solve: first position of each tile (nparts + 1
-                          // entries; nullptr: tiles of tile_rows positions)
+    // partitioned solve, on the sliced copy (solve_parts.cu; vals holds its
+    // values, idx its columns)
+    const int* part_ptr;  // first position of each part (nparts + 1)
+    const int* part_row;  // lowest row of each part
     int nparts;
+    int max_part;         // longest part
+    const int4* grp;      // descriptor of each row group
+    const int* grp_ptr;   // first group of each part (nparts + 1)
+    const void* dinv;     // 1/d(i) by position (nullptr: unit diagonal)
     // FP64 accumulation of the published values (the FP32 solves of the
     // refined solve): xacc[i][c] = v (acc_first) or xacc[i][c] += v.
     // nullptr: off.  The copying forms then skip their store to x.
@@ -112,18 +118,22 @@ cudaError_t launch_prep_column(bool f64, const SolveParams& p, const ColumnParam
 cudaError_t launch_column_k1(bool f64, int lanes, const SolveParams& p, const ColumnParams& c,
                              int grid, int block, cudaStream_t s);
 int column_blocks_per_sm(bool f64, int lanes, bool cmap, int block);
-// Blocked self-scheduled solve on the level- or part-ordered copy
-// (solve_blocked.cu): a block per tile of tile_rows consecutive positions,
-// in-tile dependencies through shared memory (tile_rows * element size at
-// most the device's opt-in shared memory per block, minus 128 B).
-// cluster in {1, 2, 4, 8}: clusters of that many blocks take consecutive
-// tiles together and read each other's tiles in distributed shared memory;
-// grid must then be a multiple of cluster.
+// Blocked self-scheduled solve on the level-ordered copy (solve_blocked.cu): a
+// block per tile of tile_rows consecutive positions, in-tile dependencies
+// through shared memory (tile_rows * element size at most 48 KB).
 cudaError_t launch_blocked_k1(bool f64, int lanes, const SolveParams& p, int tile_rows, int grid,
-                              int block, cudaStream_t s, int cluster = 1);
+                              int block, cudaStream_t s);
 // Blocks of one launch that can be resident at once (0: the shape cannot run).
-int blocked_resident_blocks(bool f64, int lanes, int cluster, int block, int tile_rows,
-                            int num_sms);
+int blocked_resident_blocks(bool f64, int lanes, int block, int tile_rows, int num_sms);
+// Partitioned solve on the sliced copy (solve_partitioned.cu): a block per part
+// of at most p.max_part positions (p.max_part * element size at most the
+// device's opt-in shared memory per block, minus 128 B).  cluster in
+// {1, 2, 4, 8}: clusters of that many blocks take consecutive parts together
+// and read each other's parts in distributed shared memory; grid must then be
+// a multiple of cluster.
+cudaError_t launch_part_k1(bool f64, int lanes, const SolveParams& p, int grid, int block,
+                           int cluster, cudaStream_t s);
+int part_resident_blocks(bool f64, int lanes, int cluster, int block, int part_rows, int num_sms);
 // Resident blocks per SM of the level-ordered-copy form of self_solve_k1.
 int self_perm_blocks_per_sm(bool f64, int lanes, int block);
 
@@ -151,16 +161,56 @@ cudaError_t launch_part_depth_keys(int np, int maxdepth, const int* pstart, cons
 // piece[p] = index of part p among the parts of its block.
 cudaError_t launch_part_piece(int np, const int* pstart, const int* bscan, const int* bstart,
                               const int* pscan, int* piece, cudaStream_t s);
-// size[r] = rows of part horder[r]; *maxsize = max (zeroed by the caller).
 // key[p] = slack of part p's block + piece[p] * levels per piece of the block.
 cudaError_t launch_part_alap_keys(int np, int maxdepth, const int* pstart, const int* bscan,
                                   const int* bstart, const int* pscan, const int* depth,
                                   const int* piece, int* key, cudaStream_t s);
-cudaError_t launch_part_sizes(int np, const int* horder, const int* pstart, int* size,
-                              int* maxsize, cudaStream_t s);
+// size[r] = rows and row[r] = lowest row of part horder[r]; *maxsize = max
+// (zeroed by the caller).
+cudaError_t launch_part_sizes(int n, int np, bool upper, const int* horder, const int* pstart,
+                              int* size, int* row, int* maxsize, cudaStream_t s);
 // key[k] = prank[part of row jlev[k]].
 cudaError_t launch_row_part_keys(int n, const int* jlev, bool upper, const int* pscan,
                                  const int* prank, int* key, cudaStream_t s);
+// Row groups and slices of the part order (position k holds row qord[k]).
+// flag[k] = 1 where a run starts: another level than position k - 1 (the part
+// starts are flagged by launch_part_flag_starts).
+cudaError_t launch_run_flags(int n, const int* qord, const int* lev, int* flag, cudaStream_t s);
+cudaError_t launch_part_flag_starts(int np, const int* part_ptr, int* flag, cudaStream_t s);
+// flag[k] = 1 at every R-th position of its run (rscan, rstart: the exclusive
+// scan of the run flags and the run starts); flag and rscan must not overlap.
+cudaError_t launch_group_flags(int n, int R, const int* rscan, const int* rstart, int* flag,
+                               cudaStream_t s);
+// grp_ptr[j] = gscan[part_ptr[j]], j = 0 .. np (gscan[n] = number of groups).
+cudaError_t launch_part_groups(int np, const int* part_ptr, const int* gscan, int* grp_ptr,
+                               cudaStream_t s);
+// Pattern of one direction and its part order, for the slicing kernels.
+struct SliceParams {
+    int n;
+    const int* ptr;       // CSR of the direction
+    const int* idx;
+    const int* vmap;      // nullptr: entry q has value vals[q]
+    int upper;
+    const int* qord;      // row at every position
+    const int* qipos;     // position of every row
+    const int* part_ptr;
+    const int* part_row;
+    int nparts, max_part;
+    const int* grp_ptr;
+    int ngroups;
+    unsigned long long* status;
+};
+// Descriptor of every group (its base left 0) from the group starts gstart
+// (ngroups + 1), and the number of its slices.
+cudaError_t launch_group_shapes(const SliceParams& p, int lanes, const int* gstart, int4* grp,
+                                int* nslices, cudaStream_t s);
+// grp[g].y = base[g].
+cudaError_t launch_group_bases(int ngroups, const int* base, int4* grp, cudaStream_t s);
+// Slices of every group: columns (nullptr: values only), values and 1/d(i)
+// (dinv nullptr: unit diagonal, values as they are).
+cudaError_t launch_fill_slices(bool f64, const SliceParams& p, int lanes, const int4* grp,
+                               const void* vals, int* cols, void* out, void* dinv,
+                               cudaStream_t s);
 
 // ---- level-ordered copy (permute.cu)
 // lens[k] = length of row jlev[k].

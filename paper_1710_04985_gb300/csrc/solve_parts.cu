@@ -6,10 +6,10 @@
 // part lies in the part itself or in an earlier part of the same run.  The
 // copy lists the parts one after another and, inside a part, its rows by
 // level (Sec. 4.1), then row; every column index is renumbered to its
-// position in that order.  A dependency then points to an earlier position,
+// position in that order, or in its part (the sliced copy, below).  A dependency then points to an earlier position,
 // one inside the part to a row of a lower level of the same part.  The
-// blocked self-scheduled kernel (solve_blocked.cu) runs on this copy with one
-// part per tile: a thread block holds its part's unknowns in shared memory,
+// partitioned kernel (solve_partitioned.cu) runs on this copy, one part per
+// thread block: the block holds its part's unknowns in shared memory,
 // where dependencies inside the part are served, and waits for earlier parts
 // through the published values as in Alg. 3.  On a structured grid in natural
 // order a part is a slab of whole grid lines, so the dependency hops along
@@ -171,15 +171,17 @@ __global__ void part_alap_keys_k(int np, int maxdepth, const int* __restrict__ p
     }
 }
 
-// size[r] = rows of the part handed out r-th; atomic max of the sizes.
-__global__ void part_sizes_k(int np, const int* __restrict__ horder,
-                             const int* __restrict__ pstart, int* size, int* maxsize) {
+// size[r] and row[r] = rows and lowest row of the part handed out r-th; atomic
+// max of the sizes.
+__global__ void part_sizes_k(int n, int np, int upper, const int* __restrict__ horder,
+                             const int* __restrict__ pstart, int* size, int* row, int* maxsize) {
     int m = 0;
     for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < np;
          r += (long long)gridDim.x * blockDim.x) {
         const int p = horder[r];
         const int s = pstart[p + 1] - pstart[p];
         size[r] = s;
+        row[r] = upper ? n - pstart[p + 1] : pstart[p];
         m = max(m, s);
     }
     m = __reduce_max_sync(0xffffffffu, m);
@@ -195,6 +197,164 @@ __global__ void row_part_keys_k(int n, const int* __restrict__ jlev, int upper,
         const int i = jlev[k];
         const long long t = upper ? n - 1 - i : i;
         key[k] = prank[pscan[t + 1] - 1];
+    }
+}
+
+// Runs of equal level inside a part, and groups of at most R rows of a run:
+// the rows a warp of the partitioned kernel takes at once.  Rows of one group
+// never depend on one another.
+__global__ void run_flags_k(int n, const int* __restrict__ qord, const int* __restrict__ lev,
+                            int* flag) {
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (long long)gridDim.x * blockDim.x)
+        flag[k] = (k == 0 || lev[qord[k]] != lev[qord[k - 1]]) ? 1 : 0;
+}
+
+__global__ void part_flag_starts_k(int np, const int* __restrict__ part_ptr, int* flag) {
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < np;
+         j += (long long)gridDim.x * blockDim.x)
+        flag[part_ptr[j]] = 1;
+}
+
+__global__ void group_flags_k(int n, int R, const int* __restrict__ rscan,
+                              const int* __restrict__ rstart, int* flag) {
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (long long)gridDim.x * blockDim.x)
+        flag[k] = ((int)k - rstart[rscan[k + 1] - 1]) % R == 0 ? 1 : 0;
+}
+
+__global__ void part_groups_k(int np, const int* __restrict__ part_ptr,
+                              const int* __restrict__ gscan, int* grp_ptr) {
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j <= np;
+         j += (long long)gridDim.x * blockDim.x)
+        grp_ptr[j] = gscan[part_ptr[j]];
+}
+
+// ---- the sliced copy
+// What the partitioned kernel reads (one copy per sub-warp width W).  A group
+// (at most 32/W rows of one level of one part) is stored as slices of 32
+// slots, slot = lane of the warp that solves it, so that every load of an
+// entry is coalesced and needs nothing but the group's descriptor
+//   { first position, first slice, X, I << 12 | span << 6 | rows }.
+// Lane sl of a row holds the row's entries sl, sl + W, ... in fold order, the
+// diagonal left out (it comes last and is kept as 1/d(i) by position).  The
+// first X slices hold entries of earlier parts (a column is a position, -1: no
+// entry), the next I slices entries of the part itself (a column is the offset
+// of the unknown in the part; no entry: max_part, a word that reads 0, with
+// value 0).  An entry of an earlier part never follows one of the part itself
+// in a lane's order, because parts are runs of consecutive rows and rows fold
+// farthest dependency first.  span: the most lanes of a row that hold entries
+// (at least 1).
+__device__ __forceinline__ int part_of_group(const SliceParams& p, int g) {
+    int lo = 0, hi = p.nparts - 1;  // last part whose first group is <= g
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.grp_ptr[mid] <= g) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Row of this lane group in fold order: entries t = 0 .. m - 1 at CSR entry
+// upper ? q0 - t : q0 + t, the diagonal (if stored) left out.
+struct FoldRow {
+    int i, q0, m, len;
+};
+__device__ __forceinline__ FoldRow fold_row(const SliceParams& p, int k, bool has) {
+    FoldRow r = {-1, 0, 0, 0};
+    if (!has) return r;
+    r.i = p.qord[k];
+    const int beg = p.ptr[r.i], end = p.ptr[r.i + 1];
+    r.len = end - beg;
+    r.q0 = p.upper ? end - 1 : beg;
+    r.m = r.len;
+    if (r.len > 0 && p.idx[p.upper ? beg : end - 1] == r.i) --r.m;
+    return r;
+}
+
+template <int W>
+__global__ void group_shapes_k(SliceParams p, const int* __restrict__ gstart, int4* grp,
+                               int* nslices) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, grow = lane / W, sl = lane % W;
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < p.ngroups;
+         g += warps) {
+        const int j = part_of_group(p, (int)g);
+        const int r0 = p.part_row[j], r1 = r0 + (p.part_ptr[j + 1] - p.part_ptr[j]);
+        const int k0 = gstart[g], cnt = gstart[g + 1] - k0;
+        const FoldRow r = fold_row(p, k0 + grow, grow < cnt);
+        int ext = 0, all = 0;
+        for (int t = sl; t < r.m; t += W, ++all) {
+            const int c = p.idx[p.upper ? r.q0 - t : r.q0 + t];
+            if (c < r0 || c >= r1) {
+                if (ext != all) report(p.status, r.i, kCodeInternal);  // not a prefix
+                ++ext;
+            }
+        }
+        const int X = __reduce_max_sync(FULL, ext);
+        const int I = __reduce_max_sync(FULL, all - ext);
+        int span = W == 1 ? 1 : __reduce_max_sync(FULL, r.m < W ? r.m : W);
+        if (span < 1) span = 1;
+        if (lane == 0) {
+            grp[g] = make_int4(k0, 0, X, (I << 12) | (span << 6) | cnt);
+            nslices[g] = X + I;
+        }
+    }
+}
+
+__global__ void group_bases_k(int ngroups, const int* __restrict__ base, int4* grp) {
+    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < ngroups;
+         g += (long long)gridDim.x * blockDim.x)
+        grp[g].y = base[g];
+}
+
+// A warp per group writes the group's slices and the 1/d(i) of its rows; checks
+// that every entry names an earlier position outside the group.
+template <typename T, int W>
+__global__ void fill_slices_k(SliceParams p, const int4* __restrict__ grp,
+                              const T* __restrict__ vals, int* cols, T* out, T* dinv) {
+    const int lane = threadIdx.x & 31, grow = lane / W, sl = lane % W;
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < p.ngroups;
+         g += warps) {
+        const int j = part_of_group(p, (int)g);
+        const int p0 = p.part_ptr[j];
+        const int r0 = p.part_row[j], r1 = r0 + (p.part_ptr[j + 1] - p0);
+        const int4 d = grp[g];
+        const int cnt = d.w & 63, I = d.w >> 12, k = d.x + grow;
+        const FoldRow r = fold_row(p, k, grow < cnt);
+        T di = T(1);
+        if (dinv && r.len > 0) {
+            const int qd = p.upper ? r.q0 - r.m : r.q0 + r.m;  // the diagonal folds last
+            di = T(1) / vals[p.vmap ? p.vmap[qd] : qd];
+            if (sl == 0) dinv[k] = di;
+        }
+        int t = sl;
+        long long at = (long long)d.y * 32 + lane;
+        for (int s = 0; s < d.z + I; ++s, at += 32) {
+            int c = s < d.z ? -1 : p.max_part;
+            T a = T(0);
+            if (t < r.m) {
+                const int q = p.upper ? r.q0 - t : r.q0 + t;
+                const int col = p.idx[q];
+                const bool ext = col < r0 || col >= r1;
+                if (ext == (s < d.z)) {
+                    const T v = vals[p.vmap ? p.vmap[q] : q];
+                    a = dinv ? v * di : v;
+                    t += W;
+                    if (cols) {
+                        const int pos = p.qipos[col];
+                        if (pos < 0 || pos >= d.x || (!ext && pos < p0) || (ext && pos >= p0))
+                            report(p.status, r.i, kCodeInternal);
+                        c = ext ? pos : pos - p0;
+                    }
+                }
+            }
+            if (cols) cols[at] = c;
+            out[at] = a;
+        }
+        if (t < r.m) report(p.status, r.i, kCodeInternal);  // an entry found no slice
     }
 }
 
@@ -261,10 +421,10 @@ cudaError_t launch_part_alap_keys(int np, int maxdepth, const int* pstart, const
     return cudaSuccess;
 }
 
-cudaError_t launch_part_sizes(int np, const int* horder, const int* pstart, int* size,
-                              int* maxsize, cudaStream_t s) {
+cudaError_t launch_part_sizes(int n, int np, bool upper, const int* horder, const int* pstart,
+                              int* size, int* row, int* maxsize, cudaStream_t s) {
     if (np <= 0) return cudaSuccess;
-    SPTRSV_LAUNCH(part_sizes_k, np, np, horder, pstart, size, maxsize);
+    SPTRSV_LAUNCH(part_sizes_k, np, n, np, upper ? 1 : 0, horder, pstart, size, row, maxsize);
     return cudaSuccess;
 }
 
@@ -273,6 +433,84 @@ cudaError_t launch_row_part_keys(int n, const int* jlev, bool upper, const int* 
     if (n <= 0) return cudaSuccess;
     SPTRSV_LAUNCH(row_part_keys_k, n, n, jlev, upper ? 1 : 0, pscan, prank, key);
     return cudaSuccess;
+}
+
+cudaError_t launch_run_flags(int n, const int* qord, const int* lev, int* flag, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    SPTRSV_LAUNCH(run_flags_k, n, n, qord, lev, flag);
+    return cudaSuccess;
+}
+
+cudaError_t launch_part_flag_starts(int np, const int* part_ptr, int* flag, cudaStream_t s) {
+    if (np <= 0) return cudaSuccess;
+    SPTRSV_LAUNCH(part_flag_starts_k, np, np, part_ptr, flag);
+    return cudaSuccess;
+}
+
+cudaError_t launch_group_flags(int n, int R, const int* rscan, const int* rstart, int* flag,
+                               cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    SPTRSV_LAUNCH(group_flags_k, n, n, R, rscan, rstart, flag);
+    return cudaSuccess;
+}
+
+cudaError_t launch_part_groups(int np, const int* part_ptr, const int* gscan, int* grp_ptr,
+                               cudaStream_t s) {
+    SPTRSV_LAUNCH(part_groups_k, (long long)np + 1, np, part_ptr, gscan, grp_ptr);
+    return cudaSuccess;
+}
+
+static int warps_grid(long long warps) {  // 8 warps a block
+    const long long g = (warps + 7) / 8;
+    return g < 1 ? 1 : (g > 16384 ? 16384 : (int)g);
+}
+
+cudaError_t launch_group_shapes(const SliceParams& p, int lanes, const int* gstart, int4* grp,
+                                int* nslices, cudaStream_t s) {
+    const int g = warps_grid(p.ngroups);
+#define SPTRSV_SHAPES(W) group_shapes_k<W><<<g, 256, 0, s>>>(p, gstart, grp, nslices)
+    switch (lanes) {
+        case 1: SPTRSV_SHAPES(1); break;
+        case 2: SPTRSV_SHAPES(2); break;
+        case 4: SPTRSV_SHAPES(4); break;
+        case 8: SPTRSV_SHAPES(8); break;
+        case 16: SPTRSV_SHAPES(16); break;
+        case 32: SPTRSV_SHAPES(32); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef SPTRSV_SHAPES
+    return cudaGetLastError();
+}
+
+cudaError_t launch_group_bases(int ngroups, const int* base, int4* grp, cudaStream_t s) {
+    SPTRSV_LAUNCH(group_bases_k, ngroups, ngroups, base, grp);
+    return cudaSuccess;
+}
+
+template <typename T>
+static cudaError_t fill_t(const SliceParams& p, int lanes, const int4* grp, const void* vals,
+                          int* cols, void* out, void* dinv, cudaStream_t s) {
+    const int g = warps_grid(p.ngroups);
+#define SPTRSV_FILL(W) \
+    fill_slices_k<T, W><<<g, 256, 0, s>>>(p, grp, (const T*)vals, cols, (T*)out, (T*)dinv)
+    switch (lanes) {
+        case 1: SPTRSV_FILL(1); break;
+        case 2: SPTRSV_FILL(2); break;
+        case 4: SPTRSV_FILL(4); break;
+        case 8: SPTRSV_FILL(8); break;
+        case 16: SPTRSV_FILL(16); break;
+        case 32: SPTRSV_FILL(32); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef SPTRSV_FILL
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fill_slices(bool f64, const SliceParams& p, int lanes, const int4* grp,
+                               const void* vals, int* cols, void* out, void* dinv,
+                               cudaStream_t s) {
+    return f64 ? fill_t<double>(p, lanes, grp, vals, cols, out, dinv, s)
+               : fill_t<float>(p, lanes, grp, vals, cols, out, dinv, s);
 }
 
 #undef SPTRSV_LAUNCH
