@@ -675,6 +675,24 @@ cudaError_t launch_inverse_perm(const int* perm, int n, int* ipos, cudaStream_t 
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------------ row lengths
+__global__ void max_length_k(int n, const int* __restrict__ ptr, int* most) {
+    int m = 0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x)
+        m = max(m, ptr[i + 1] - ptr[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(most, m);
+}
+
+cudaError_t launch_max_length(int n, const int* ptr, int* most, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    long long g = ((long long)n + 255) / 256;
+    if (g > 608) g = 608;
+    max_length_k<<<(int)g, 256, 0, s>>>(n, ptr, most);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------ level-set check
 __global__ void verify_levels_k(int n, int nlev, const int* __restrict__ lev,
                                 const int* __restrict__ ilev, const int* __restrict__ jlev,

@@ -36,6 +36,7 @@ sptrsv_status_t cuda_fail(cudaError_t e) {
 
 struct Levels {
     int nlev = 0;
+    int max_len = 0;  // longest row
     int* lev = nullptr;
     int* ilev = nullptr;
     int* jlev = nullptr;
@@ -105,6 +106,8 @@ struct Levels {
 // Each slot costs a load in the solve; a width at which eight in nine slots are
 // empty is never the one to use.
 constexpr long long kMaxPadding = 8;
+constexpr int kSmallBlock = 512;  // threads of a solve in one block, and
+constexpr int kSmallGroups = 4;   // the row groups per level it is used for
 
 void free_slices(Levels::Slices& q) {
     cudaFree(q.grp);
@@ -202,7 +205,7 @@ struct sptrsv_plan_s {
     int* tptr = nullptr;
     int* tidx = nullptr;
     int* tmap = nullptr;
-    int* counters = nullptr;  // [0] ticket, [1] level count
+    int* counters = nullptr;  // [0] ticket, [1] level count, [2] longest row
     unsigned long long* status = nullptr;
     void* bcopy = nullptr;
     size_t bcopy_bytes = 0;
@@ -300,7 +303,7 @@ sptrsv_status_t take_status(sptrsv_plan_t P, cudaStream_t s, int* row) {
 
 sptrsv_status_t sweep_levels(sptrsv_plan_t P, const int* ptr, const int* idx, bool upper,
                              Levels& L, int* nlev_out, cudaStream_t s);
-sptrsv_status_t level_sets(sptrsv_plan_t P, Levels& L, int nlev, cudaStream_t s);
+sptrsv_status_t level_sets(sptrsv_plan_t P, const int* ptr, Levels& L, int nlev, cudaStream_t s);
 
 // Levels by Kahn's algorithm (Sec. 4.4.1): dptr/didx is the CSR of the
 // transpose of the system (row i lists the rows that depend on i).  The
@@ -415,7 +418,7 @@ sptrsv_status_t build_levels(sptrsv_plan_t P, const int* ptr, const int* idx, bo
         }
         ST(sweep_levels(P, ptr, idx, upper, L, &nlev, s));
     }
-    return level_sets(P, L, nlev, s);
+    return level_sets(P, ptr, L, nlev, s);
 }
 
 // Levels by the sync-free sweep (analysis.cu).  Writes L.lev and *nlev;
@@ -452,7 +455,7 @@ sptrsv_status_t sweep_levels(sptrsv_plan_t P, const int* ptr, const int* idx, bo
 // Level sets from L.lev (Sec. 4.1): histogram, exclusive scan to ilev, a
 // stable radix sort of the rows by level to jlev (ascending rows inside a
 // level), a self-check, and the inverse permutation ipos.  Synchronises s.
-sptrsv_status_t level_sets(sptrsv_plan_t P, Levels& L, int nlev, cudaStream_t s) {
+sptrsv_status_t level_sets(sptrsv_plan_t P, const int* ptr, Levels& L, int nlev, cudaStream_t s) {
     const int n = P->n;
     int row = -1;
     L.nlev = nlev;
@@ -479,6 +482,10 @@ sptrsv_status_t level_sets(sptrsv_plan_t P, Levels& L, int nlev, cudaStream_t s)
         e = radix_sort_values(L.lev, nullptr, n, bits_for(nlev - 1), L.jlev, k_a, v_a, k_b, v_b,
                               hist, hist_scan, P->status, s);
     if (e == cudaSuccess) e = launch_verify_levels(n, nlev, L.lev, L.ilev, L.jlev, P->status, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(P->counters + 2, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = launch_max_length(n, ptr, P->counters + 2, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&L.max_len, P->counters + 2, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) {
         L.h_ilev.resize((size_t)nlev + 1);
         e = cudaMemcpyAsync(L.h_ilev.data(), L.ilev, sizeof(int) * (size_t)(nlev + 1),
@@ -778,6 +785,28 @@ int max_part_rows(sptrsv_plan_t P) {
     const int esize = P->f64 ? 8 : 4;
     const int room = P->smem_optin - 128;
     return room > esize * 32 ? (room / esize) & ~31 : 32;
+}
+
+// Whether the rows of every ticket of the self-scheduled kernel are taken as one:
+// rows of about equal length, and tickets of 32 / lanes rows that span few
+// levels on average.  (In-place solves before and after, us: 7-point 128^3 570 ->
+// 514, 27-point 61 x 47 x 53 467 -> 380, 5-point 120 x 130 249 -> 239.)
+bool rows_alike(sptrsv_plan_t P, const Levels& L, int lanes) {
+    return (long long)L.max_len * P->n <= 2ll * P->nnz + 2ll * P->n &&
+           32ll * L.nlev <= 3ll * lanes * P->n;
+}
+
+// Whether a single-RHS solve of the in-place or level-ordered form runs in one
+// block with its unknowns in shared memory: they must fit there, rows must be
+// alike, and an average level must hold few enough row groups (32 / lanes rows)
+// for one SM.  (5-point grids, plan defaults, us: 64 x 64 FP64 123 -> 82 and FP32
+// 115 -> 56 at two groups per level; 120 x 130 FP64 249 -> 196 at four; 160 x 160
+// FP32 299 -> 194 at five.  The 7-point 20 x 18 x 22 grid, 17 groups per level:
+// 71 us on the whole GPU, 170 in one block.)
+bool small_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes) {
+    if ((f64 ? 8ll : 4ll) * P->n > P->smem_optin - 128 || !rows_alike(P, L, lanes)) return false;
+    // FP32 rows take half the time: no FP64 unit to wait for
+    return (long long)P->n * lanes <= 32ll * kSmallGroups * (f64 ? 1 : 2) * L.nlev;
 }
 
 // The part size of the next partitioned solve: the plan's setting or the
@@ -1162,6 +1191,8 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     p.diag_first = trans ? !P->upper : P->upper;
     p.unit = P->unit;
     p.jlev = L.jlev;
+    p.lev = L.lev;
+    p.rows_alike = rows_alike(P, L, lanes) ? 1 : 0;
     p.b = b;
     p.ldb = ldb;
     p.x = x;
@@ -1279,12 +1310,18 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         p.vals = f32_of_f64 ? L.pvals32 : L.pvals;
         p.xp = f32_of_f64 ? L.xp32 : L.xp;
         p.prescaled = P->unit ? 0 : 1;
-        CK(launch_prep_self(f64, P->n, 1, p.xp, 1, nullptr, 0, nullptr, P->counters,
-                            P->num_sms * 8, s));
+        const bool small = !blocked && small_solve(P, L, f64, lanes);
+        if (!small)
+            CK(launch_prep_self(f64, P->n, 1, p.xp, 1, nullptr, 0, nullptr, P->counters,
+                                P->num_sms * 8, s));
         const int R = 32 / lanes;
         const long long tickets = ((long long)P->n + R - 1) / R;
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
-        if (blocked) {
+        if (small) {
+            ST(prof_begin(P, s));
+            CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
+            ST(prof_end(P, s));
+        } else if (blocked) {
             const long long tiles = ((long long)P->n + P->tile_rows - 1) / P->tile_rows;
             long long grid = blocked_resident_blocks(f64, lanes, block, P->tile_rows, P->num_sms);
             if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
@@ -1295,7 +1332,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             ST(prof_end(P, s));
         } else {
             long long grid =
-                (long long)self_perm_blocks_per_sm(f64, lanes, block) * P->num_sms;
+                (long long)self_k1_blocks_per_sm(f64, lanes, false, true, block) * P->num_sms;
             if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
             if (grid > want_blocks) grid = want_blocks;
             if (grid < 1) grid = 1;
@@ -1303,7 +1340,12 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             CK(launch_self_k1(f64, lanes, p, (int)grid, block, s));
             ST(prof_end(P, s));
         }
-        launches = 2;
+        launches = small ? 1 : 2;
+    } else if (algo == SPTRSV_ALGO_SELF && !mrhs && small_solve(P, L, f64, lanes)) {
+        ST(prof_begin(P, s));
+        CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
+        ST(prof_end(P, s));
+        launches = 1;
     } else {
         const size_t esize = f64 ? sizeof(double) : sizeof(float);
         void* bcopy = nullptr;

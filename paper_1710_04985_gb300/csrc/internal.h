@@ -19,6 +19,8 @@ struct SolveParams {
     int diag_first;       // upper-triangular pattern: diagonal is a row's first entry
     int unit;
     const int* jlev;      // rows in level order
+    const int* lev;       // level of every row
+    int rows_alike;       // every ticket's rows are taken as one (solve_self.cu)
     const void* b;
     long long ldb;
     void* x;
@@ -134,8 +136,13 @@ int blocked_resident_blocks(bool f64, int lanes, int block, int tile_rows, int n
 cudaError_t launch_part_k1(bool f64, int lanes, const SolveParams& p, int grid, int block,
                            int cluster, cudaStream_t s);
 int part_resident_blocks(bool f64, int lanes, int cluster, int block, int part_rows, int num_sms);
-// Resident blocks per SM of the level-ordered-copy form of self_solve_k1.
-int self_perm_blocks_per_sm(bool f64, int lanes, int block);
+// Resident blocks per SM of self_solve_k1 (perm: its level-ordered-copy form).
+int self_k1_blocks_per_sm(bool f64, int lanes, bool map, bool perm, int block);
+// The whole system in one block, its unknowns in shared memory (n * element size
+// at most the device's opt-in shared memory per block, minus 128 B).  Needs no
+// prep launch: b is read before x is written, in place too.
+cudaError_t launch_self_small(bool f64, int lanes, const SolveParams& p, int block,
+                              cudaStream_t s);
 
 // ---- partitioned solve (solve_parts.cu).  Positions t are in order of
 // substitution (row t of a lower system, row n-1-t of an upper one).
@@ -270,6 +277,8 @@ cudaError_t launch_gather(const int* src, int src_len, const int* index, int m, 
                           unsigned long long* status, cudaStream_t s);
 // ipos[perm[k]] = k (perm is a permutation of 0..n-1; checked before).
 cudaError_t launch_inverse_perm(const int* perm, int n, int* ipos, cudaStream_t s);
+// *most = max(*most, longest row).
+cudaError_t launch_max_length(int n, const int* ptr, int* most, cudaStream_t s);
 // Self-check of level sets: every position of jlev holds a row of the
 // level whose segment contains it, rows strictly increase inside a segment,
 // ilev[0] = 0 and ilev[nlev] = n.  Failures are reported as internal.

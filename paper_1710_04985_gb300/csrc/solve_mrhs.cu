@@ -245,10 +245,8 @@ static int occ_mrhs(int lanes, int block) {
     return (e == cudaSuccess && nb > 0) ? nb : 1;
 }
 
-int self_k1_blocks_per_sm(bool f64, int lanes, bool map, int block);
-
 int self_blocks_per_sm(bool f64, int lanes, bool mrhs, bool map, int block) {
-    if (!mrhs) return self_k1_blocks_per_sm(f64, lanes, map, block);
+    if (!mrhs) return self_k1_blocks_per_sm(f64, lanes, map, false, block);
     if (f64) return map ? occ_mrhs<double, true>(lanes, block) : occ_mrhs<double, false>(lanes, block);
     return map ? occ_mrhs<float, true>(lanes, block) : occ_mrhs<float, false>(lanes, block);
 }

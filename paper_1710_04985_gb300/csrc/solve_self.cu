@@ -11,14 +11,27 @@
 //    a dependency costs one L2 round trip and no fence.
 //  * A row is reduced by a sub-warp of W lanes (W chosen per matrix).  The
 //    paper lets lane 0 spin and relies on warp lockstep, which sm_70 and
-//    later no longer guarantee.  Here the whole warp stays converged in one
-//    round loop: every lane issues the loads of all its entries of a chunk
-//    at once, re-polls only the pending ones each round, and a row is reduced
-//    (shuffles) and published inside the loop as soon as all its lanes are
-//    done.  Rows of one ticket may therefore depend on one another (a ticket
-//    can straddle two levels) without deadlock, and no sub-warp waits in a
-//    divergent spin that the scheduler would serialise.  Every wait is
-//    bounded.
+//    later no longer guarantee.  Here the whole warp stays converged, in one of
+//    two ways.  Rows of one level never depend on one another, so the warp waits
+//    until all their values are there, folds, reduces and publishes them as one
+//    (a ticket that straddles a few levels does so level by level).  Where the
+//    rows of a ticket differ (a long row among short ones), every row is
+//    folded and published as soon as its own values are there (rows_apart).
+//
+// What bounds it: a hop of the dependency chain, which is an L2 handshake
+// (~350 ns), the fold and lane reduction that follow the last arrival (~64 cycles
+// per FP64 instruction) and the instructions around them (4 to 5 cycles each, a
+// taken branch ~30).  The loop that polls therefore does nothing else, a row's
+// next chunk of entries is loaded before the wait for the current one, and
+// whatever does not depend on x is computed before the first wait.  A warp that
+// waits for more than a quarter of the spin limit goes on in rows_apart(), so that
+// a value that never comes holds up only the rows that depend on it.
+//
+// Measured against the kernel before (every row folded and published by itself,
+// tickets of any levels in one round loop), plan defaults, FP64, us: 7-point
+// 61 x 47 x 53 in place 205 -> 182 and its adjoint 210 -> 182, 27-point of that
+// size 467 -> 381, 128^3 ILU(0) L 570 -> 548; general matrix of 150001 rows 5656 ->
+// 5300 and its adjoint 5688 -> 5231 (16 lanes; 32 lanes 4858 -> 4810).
 #include "internal.h"
 
 namespace sptrsv {
@@ -59,6 +72,261 @@ cudaError_t launch_prep_self(bool f64, int n, int nrhs, void* x, long long ldx, 
 }
 
 
+namespace {
+
+constexpr int kMaxSelfBlock = 512;  // larger blocks run as several of this size
+constexpr int kSelfHot = 64;        // polls of one wait before the warp backs off
+
+__device__ __forceinline__ double lds_relaxed(const double* p) { return *(const volatile double*)p; }
+__device__ __forceinline__ float lds_relaxed(const float* p) { return *(const volatile float*)p; }
+
+// One row of a ticket as its lanes see it.
+template <typename T>
+struct Row {
+    int i, beg, end, lev;
+    long long k;
+    bool has;
+    T dinv, sum;
+    double xbase;  // refinement: the solution the row's value is added to
+};
+
+template <typename T, int W, bool PERM>
+__device__ __forceinline__ Row<T> take_row(const SolveParams& p, long long k) {
+    Row<T> r;
+    r.k = k;
+    r.has = k < p.n;
+    r.i = r.beg = r.end = r.lev = 0;
+    r.dinv = T(1);
+    r.sum = T(0);
+    r.xbase = 0.0;
+    if (r.has) {
+        r.i = p.jlev[k];
+        r.beg = p.ptr[PERM ? k : r.i];
+        r.end = p.ptr[(PERM ? k : r.i) + 1];
+        if (W < 32) r.lev = p.lev[r.i];
+    }
+    return r;
+}
+
+// Everything of a row that does not depend on x: SLFR computes 1/d(i) up front
+// too; the row is scaled by it, so x(i) = b(i)/d(i) - sum of (a_ij/d(i)) x(j) and
+// only the FMA fold and the lane reduction remain once the last value is there.
+template <typename T, int W, bool MAP>
+__device__ __forceinline__ void start_row(const SolveParams& p, Row<T>& r, int sl) {
+    if (r.has && sl == 0) {
+        const T* __restrict__ vals = (const T*)p.vals;
+        if (!p.unit) {
+            const int q = p.diag_first ? r.beg : r.end - 1;
+            const T d = vals[MAP ? p.vmap[q] : q];
+            r.dinv = p.prescaled ? d : T(1) / d;  // a pre-scaled copy holds 1/d(i)
+        }
+        r.sum = ((const T*)p.b)[(long long)r.i * p.ldb];
+        if (!p.unit) r.sum *= r.dinv;
+        r.xbase = accumulate_base(p, r.i, 0);
+    }
+    if (W > 1 && !p.unit && !p.prescaled)
+        r.dinv = __shfl_sync(0xffffffffu, r.dinv, (threadIdx.x & 31) / W * W);
+}
+
+// Entries q0, q0 + W, ... of a row in fold order: the unknown to wait for (-1:
+// none, the diagonal included) and the scaled value (0).
+template <typename T, int W, bool MAP, bool PERM, int E>
+__device__ __forceinline__ void load_entries(const SolveParams& p, const Row<T>& r, int q0,
+                                             int (&c)[E], T (&a)[E]) {
+    const T* __restrict__ vals = (const T*)p.vals;
+    // every form folds farthest dependency first: a lower row in storage order,
+    // an upper row from its last entry back (the copies already store it so)
+    const bool rvs = !PERM && p.diag_first;
+    const int self = PERM ? (int)r.k : r.i;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int q = q0 + e * W;
+        c[e] = -1;
+        a[e] = T(0);
+        if (q < r.end) {
+            const int pq = rvs ? r.beg + r.end - 1 - q : q;
+            c[e] = p.idx[pq];
+            a[e] = vals[MAP ? p.vmap[pq] : pq];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (c[e] == self) {
+            c[e] = -1;
+            a[e] = T(0);
+        }
+}
+
+// Scales the loaded values of a row that is not pre-scaled (slots that no lane
+// uses are branched around: an FP64 multiply takes 64 cycles).
+template <typename T, int E>
+__device__ __forceinline__ void scale_entries(const SolveParams& p, T dinv, const int (&c)[E],
+                                              T (&a)[E]) {
+    if (p.unit || p.prescaled) return;
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (__any_sync(0xffffffffu, c[e] >= 0)) {
+            if (c[e] >= 0) a[e] *= dinv;
+        }
+}
+
+// Whether the warp takes the rows of a ticket as one, where the matrix as a
+// whole does not say so (SolveParams::rows_alike): equally many chunks of
+// entries, lengths within a factor of about two (unless there are only two
+// rows), and at most kLevels levels.  A general matrix of 20001 rows with 4 lanes
+// per row (mean row 14 entries, longest 900) took 2.36 ms with every ticket as
+// one and 1.09 ms with its rows apart.
+template <int W>
+__device__ __forceinline__ bool alike(bool has, int len, int lev) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int kLevels = 4;
+    const int most = __reduce_max_sync(FULL, has ? len : 0);
+    const int least = __reduce_min_sync(FULL, has ? len : 0x7fffffff);
+    const int top = __reduce_max_sync(FULL, has ? lev : -1);
+    const int low = __reduce_min_sync(FULL, has ? lev : 0x7fffffff);
+    if (top - low >= kLevels) return false;
+    if ((most + W * kChunk - 1) / (W * kChunk) != (least + W * kChunk - 1) / (W * kChunk))
+        return false;
+    return W >= 16 || most <= 2 * least + 2;
+}
+
+}  // namespace
+
+// The rows of ticket t one by one: every row is folded as its values come and
+// published by itself.  Gives up (false) after `budget` polls without an end;
+// again: rows that are published already are skipped.
+template <typename T, int W, bool MAP, bool PERM, bool SMALL>
+__device__ __noinline__ bool rows_apart(const SolveParams& p, long long t, T* xs, bool again,
+                                        long long budget) {
+    constexpr int R = 32 / W;
+    constexpr int E = kChunk;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int grp = lane / W;
+    const int sl = lane - grp * W;
+    const unsigned gmask = group_mask<W>(lane);
+    T* xpub = SMALL ? xs : PERM ? (T*)p.xp : (T*)p.x;
+    const long long ldp = (SMALL || PERM) ? 1 : p.ldx;
+    Row<T> r = take_row<T, W, PERM>(p, t * R + grp);
+    start_row<T, W, MAP>(p, r, sl);
+    const int span = warp_span<W>(r.has, r.end - r.beg);
+    const long long own = (PERM ? r.k : (long long)r.i) * ldp;
+    auto look = [&](long long at) -> T {
+        return SMALL ? lds_relaxed(xpub + at) : ld_relaxed(xpub + at);
+    };
+    bool published = !r.has || (again && !Marker<T>::pending(look(own)));
+    int q0 = r.beg + sl, c[E];
+    T a[E], v[E];
+    unsigned live = 0, pend = 0;
+    auto load_chunk = [&]() {
+        load_entries<T, W, MAP, PERM, E>(p, r, q0, c, a);
+        live = pend = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            v[e] = T(0);
+            if (c[e] >= 0) {
+                live |= 1u << e;
+                v[e] = look((long long)c[e] * ldp);
+            }
+        }
+        if (!p.unit && !p.prescaled) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (live & (1u << e)) a[e] *= r.dinv;
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if ((live & (1u << e)) && Marker<T>::pending(v[e])) pend |= 1u << e;
+    };
+    bool lane_done = published || q0 >= r.end;
+    if (!lane_done) load_chunk();
+    long long waits = 0, total = 0;
+    unsigned ns = 32;
+    while (true) {
+        if (!lane_done && pend == 0) {  // fold a complete chunk in fold order
+            if (live) r.sum = fold_chunk(r.sum, a, v, live);
+            q0 += W * E;
+            if (q0 >= r.end)
+                lane_done = true;
+            else
+                load_chunk();
+        }
+        const unsigned done = __ballot_sync(FULL, lane_done);
+        const bool fresh = !published && (done & gmask) == gmask;
+        if (__any_sync(FULL, fresh)) {
+            const T tot = group_sum_span<W>(r.sum, FULL, span);
+            if (fresh && sl == 0 && r.i != p.withhold) {
+                const T val = publishable(tot);
+                if (SMALL)
+                    *(volatile T*)(xpub + own) = val;
+                else
+                    st_relaxed(xpub + own, val);
+                if (p.xacc)
+                    accumulate_with(p, r.i, 0, val, r.xbase);
+                else if (PERM || SMALL)
+                    ((T*)p.x)[(long long)r.i * p.ldx] = val;
+            }
+        }
+        published = published || fresh;
+        if (__all_sync(FULL, published)) return true;
+        if (__any_sync(FULL, !lane_done && pend == 0)) continue;  // fold first
+        if (!__any_sync(FULL, pend != 0)) {
+            waits = 0;
+            ns = 32;
+            continue;
+        }
+        const unsigned before = pend;
+        do {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (pend & (1u << e)) v[e] = look((long long)c[e] * ldp);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if ((pend & (1u << e)) && !Marker<T>::pending(v[e])) pend &= ~(1u << e);
+            if (++total > budget) return false;
+            if (++waits >= p.spin.limit) {
+                if (pend) {
+                    report(p.status, r.i, kCodeTimeout);
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (pend & (1u << e)) v[e] = Marker<T>::canonical_nan();
+                    pend = 0;
+                }
+                waits = 0;
+                break;
+            }
+            if (__any_sync(FULL, pend != before)) break;
+            if (waits >= p.spin.hot) {
+                __nanosleep(ns);
+                ns = ns < p.spin.max_ns ? ns * 2 : p.spin.max_ns;
+            }
+        } while (true);
+    }
+}
+
+// A value that ticket t's rows wait for has not come for long.  The rows of the
+// ticket this warp also holds must not wait for it where they do not need it:
+// turns of a few polls for both, until both are done or the polls reach the spin
+// limit, then one after the other to its end.  Returns (in lane 0) the warp's
+// next ticket.
+template <typename T, int W, bool MAP, bool PERM, bool SMALL>
+__device__ __noinline__ int stuck_rows(const SolveParams& p, long long t, int tn, int* ticket,
+                                       T* xs) {
+    constexpr int kTurn = 256;
+    constexpr long long kNoEnd = 1ll << 62;  // the wait ends by the spin limit
+    const long long t2 = __shfl_sync(0xffffffffu, tn, 0);
+    const bool held = !SMALL && t2 * (32 / W) < p.n;
+    bool done = false, done2 = !held;
+    for (long long polls = 0; !(done && done2) && polls < p.spin.limit; polls += kTurn) {
+        if (!done) done = rows_apart<T, W, MAP, PERM, SMALL>(p, t, xs, true, kTurn);
+        if (!done2) done2 = rows_apart<T, W, MAP, PERM, SMALL>(p, t2, xs, true, kTurn);
+    }
+    if (!done) rows_apart<T, W, MAP, PERM, SMALL>(p, t, xs, true, kNoEnd);
+    if (!done2) rows_apart<T, W, MAP, PERM, SMALL>(p, t2, xs, true, kNoEnd);
+    if (held && (threadIdx.x & 31) == 0) tn = atomicAdd(ticket, 1);
+    return tn;
+}
+
 // PERM: the pattern is the plan's level-ordered copy (SPTRSV_ALGO_SELF_PERMUTED):
 // row position k of jlev holds the entries of row jlev[k] in fold order (an
 // upper row's last entry first), with column indices renumbered to positions
@@ -67,260 +335,214 @@ cudaError_t launch_prep_self(bool f64, int n, int nrhs, void* x, long long ldx, 
 // the array that is polled) and stored to x(jlev[k]) for the caller.  The
 // arithmetic and its order are those of the unpermuted kernel, so both give
 // bitwise identical results for the same sub-warp width.
-template <typename T, int W, bool MAP, bool PERM>
-__global__ void __launch_bounds__(1024) self_solve_k1(SolveParams p) {
+//
+// SMALL: one block solves the whole system with its unknowns in shared memory
+// (a hop is a shared-memory poll instead of an L2 handshake), for systems that
+// fit there and whose levels are too narrow to occupy more than one SM.
+template <typename T, int W, bool MAP, bool PERM, bool SMALL>
+__global__ void __launch_bounds__(kMaxSelfBlock, 1)
+    self_solve_k1(const __grid_constant__ SolveParams p) {
+    extern __shared__ __align__(16) unsigned char self_smem[];
+    __shared__ int s_next;
     constexpr int R = 32 / W;
     constexpr int E = kChunk;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int grp = lane / W;
     const int sl = lane - grp * W;
-    const unsigned gmask = group_mask<W>(lane);
-    const T* __restrict__ vals = (const T*)p.vals;
-    const T* b = (const T*)p.b;
+    T* xs = (T*)self_smem;
     T* x = (T*)p.x;
-    T* xpub = PERM ? (T*)p.xp : x;  // the array rows publish to and wait on
-    const long long ldp = PERM ? 1 : p.ldx;
-    // Every form folds a row's entries farthest dependency first: a lower
-    // row in storage order, an upper row from its last entry back (the copies
-    // already store an upper row that way round).
-    const bool rvs = !PERM && p.diag_first;
+    T* xpub = SMALL ? xs : PERM ? (T*)p.xp : x;  // the array rows publish to and wait on
+    const long long ldp = (SMALL || PERM) ? 1 : p.ldx;
+    const long long patience = p.spin.limit / 4 + 1;
+    auto look = [&](int c) -> T {
+        return SMALL ? lds_relaxed(xpub + c) : ld_relaxed(xpub + (long long)c * ldp);
+    };
+    if (SMALL) {
+        for (int k = threadIdx.x; k < p.n; k += blockDim.x) xs[k] = Marker<T>::pending_value();
+        if (threadIdx.x == 0) s_next = 0;
+        __syncthreads();
+    }
+    int* const ticket = SMALL ? &s_next : p.ticket;
     int t = 0;
-    if (lane == 0) t = atomicAdd(p.ticket, 1);
+    if (lane == 0) t = atomicAdd(ticket, 1);
     t = __shfl_sync(FULL, t, 0);
     while ((long long)t * R < p.n) {
         int tn = 0;
-        if (lane == 0) tn = atomicAdd(p.ticket, 1);  // next ticket, consumed after this one
-        const long long k = (long long)t * R + grp;
-        const bool has_row = k < p.n;
-        int i = 0, beg = 0, end = 0;
-        T dinv = T(1), sum = T(0);
-        double xbase = 0.0;  // refinement: the solution the row's value is added to
-        // identity of the row inside the pattern: its own column index
-        const int self_col = PERM ? (int)k : 0;
-        if (has_row) {
-            i = p.jlev[k];
-            beg = p.ptr[PERM ? k : i];
-            end = p.ptr[(PERM ? k : i) + 1];
-            if (sl == 0) {
-                // Everything that does not depend on x happens now, while the
-                // dependencies are pending (SLFR computes 1/d(i) up front too):
-                // the row is scaled by 1/d(i), so x(i) = b(i)/d(i) - sum of
-                // (a_ij/d(i)) x(j) and only the FMA fold and the lane reduction
-                // remain once the last dependency arrives.
-                if (!p.unit) {
-                    const int q = p.diag_first ? beg : end - 1;
-                    const T d = vals[MAP ? p.vmap[q] : q];
-                    dinv = p.prescaled ? d : T(1) / d;  // a pre-scaled copy holds 1/d(i)
-                }
-                sum = b[(long long)i * p.ldb];
-                if (!p.unit) sum *= dinv;
-                xbase = accumulate_base(p, i, 0);
-            }
+        if (!SMALL && lane == 0) tn = atomicAdd(ticket, 1);  // consumed after this one
+        Row<T> r = take_row<T, W, PERM>(p, (long long)t * R + grp);
+        if (R > 1 && !p.rows_alike && !alike<W>(r.has, r.end - r.beg, r.lev)) {
+            if (!rows_apart<T, W, MAP, PERM, SMALL>(p, t, xs, false, patience))
+                tn = stuck_rows<T, W, MAP, PERM, SMALL>(p, t, tn, ticket, xs);
+            if (SMALL && lane == 0) tn = atomicAdd(ticket, 1);
+            t = __shfl_sync(FULL, tn, 0);
+            continue;
         }
-        if (W > 1 && !p.unit && !p.prescaled) dinv = __shfl_sync(FULL, dinv, grp * W);
-        const int span = warp_span<W>(has_row, end - beg);
-        // ---- per-lane chunk state: entries q0 + e*W, e < E
-        int q0 = beg + sl;
-        int c[E];
+        start_row<T, W, MAP>(p, r, sl);
+        int q0 = r.beg + sl, c[E];
         T a[E], v[E];
-        unsigned live = 0, pend = 0;  // entries that count / still unpublished
-        auto load_chunk = [&]() {
-            live = pend = 0;
+        load_entries<T, W, MAP, PERM, E>(p, r, q0, c, a);
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int q = q0 + e * W;
-                c[e] = -1;
-                a[e] = T(0);
-                v[e] = T(0);
-                if (q < end) {
-                    const int pq = rvs ? beg + end - 1 - q : q;  // fold order -> storage
-                    const int cc = p.idx[pq];
-                    if (cc != (PERM ? self_col : i)) {
-                        c[e] = cc;
-                        a[e] = vals[MAP ? p.vmap[pq] : pq];
-                        live |= 1u << e;
-                    }
-                }
+        for (int e = 0; e < E; ++e) {
+            v[e] = T(0);
+            if (c[e] >= 0) v[e] = look(c[e]);
+        }
+        scale_entries(p, r.dinv, c, a);
+        const int span = warp_span<W>(r.has, r.end - r.beg);
+        const long long own = PERM ? r.k : (long long)r.i * ldp;
+        bool todo = r.has, ok = true;
+        while (true) {
+            // the rows of the lowest level that is left
+            bool act = todo;
+            if (W < 32) {
+                const int low = __reduce_min_sync(FULL, todo ? r.lev : 0x7fffffff);
+                act = todo && r.lev == low;
             }
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                if (live & (1u << e)) v[e] = ld_relaxed(xpub + (long long)c[e] * ldp);
-            if (!p.unit && !p.prescaled) {
+            while (true) {  // chunks of entries
+                const bool more = __any_sync(FULL, act && q0 + W * E < r.end);
+                // slots in use: the chunk's dead slots come after its live ones,
+                // but for the diagonal of a row whose fold order it does not end
+                unsigned slots = 0;
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    if (live & (1u << e)) a[e] *= dinv;
-            }
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                if ((live & (1u << e)) && Marker<T>::pending(v[e])) pend |= 1u << e;
-        };
-        // one lane per row: store the row's value (and x, on the copy)
-        auto publish_row = [&](T tot) {
-            const T val = publishable(tot);
-            st_relaxed(xpub + (PERM ? k : (long long)i * p.ldx), val);
-            if (p.xacc)
-                accumulate_with(p, i, 0, val, xbase);
-            else if (PERM)
-                x[(long long)i * p.ldx] = val;
-        };
-        bool lane_done = q0 >= end;
-        if (!lane_done) load_chunk();
-        bool published = !has_row;
-        long long waits = 0;
-        unsigned ns = 32;
-        while (true) {
-            if (!lane_done && pend == 0) {  // fold a complete chunk in fold order
-                sum = fold_chunk(sum, a, v, live);
-                q0 += W * E;
-                if (q0 >= end) {
-                    lane_done = true;
-                    // one lane per row: the row is complete, publish it at once
-                    // (no lane reduction to wait for)
-                    if (W == 1 && has_row && i != p.withhold) {
-                        publish_row(sum);
-                        published = true;
-                    }
-                } else {
-                    load_chunk();
+                    if (__any_sync(FULL, act && c[e] >= 0)) slots |= 1u << e;
+                int c2[E];
+                T a2[E];
+                if (more) {
+                    load_entries<T, W, MAP, PERM, E>(p, r, q0 + W * E, c2, a2);
+                    scale_entries(p, r.dinv, c2, a2);
                 }
-            }
-            const unsigned done = __ballot_sync(FULL, lane_done);
-            const bool fresh = !published && (done & gmask) == gmask;
-            if (__any_sync(FULL, fresh)) {  // FP64 is scarce on GB300: reduce only then
-                const T tot = group_sum_span<W>(sum, FULL, span);
-                if (fresh && sl == 0 && i != p.withhold) publish_row(tot);
-            }
-            published = published || fresh;
-            if (__all_sync(FULL, published)) break;
-            // A lane with a complete chunk folds it first (next round); only
-            // when every lane is done or waiting does the warp enter the tight
-            // wait, so a row of this ticket that another row waits on is
-            // never held back by the wait.
-            if (__any_sync(FULL, !lane_done && pend == 0)) continue;
-            // Tight wait: re-poll the pending entries until something arrives
-            // anywhere in the warp (one vote per poll; uniform control flow).
-            if (__any_sync(FULL, pend != 0)) {
-                const unsigned before = pend;
-                do {
+                long long polls = 0;
+                while (true) {
+                    bool pend = false;
 #pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        if (pend & (1u << e)) v[e] = ld_relaxed(xpub + (long long)c[e] * ldp);
-#pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        if ((pend & (1u << e)) && !Marker<T>::pending(v[e])) pend &= ~(1u << e);
-                    // one lane per row and this was the row's last chunk: fold
-                    // and publish now, before the warp leaves the wait
-                    if (W == 1 && !lane_done && pend == 0 && q0 + E >= end) {
-                        sum = fold_chunk(sum, a, v, live);
-                        q0 += E;
-                        lane_done = true;
-                        if (has_row && i != p.withhold) publish_row(sum);
-                        published = true;
-                    }
-                    if (++waits >= p.spin.limit) {
-                        if (pend) {
-                            report(p.status, i, kCodeTimeout);
-#pragma unroll
-                            for (int e = 0; e < E; ++e)
-                                if (pend & (1u << e)) v[e] = Marker<T>::canonical_nan();
-                            pend = 0;
+                    for (int e = 0; e < E; ++e) pend |= Marker<T>::pending(v[e]);
+                    if (!__any_sync(FULL, act && pend)) break;
+                    if (++polls > kSelfHot) {
+                        if (polls > patience) {
+                            ok = false;
+                            break;
                         }
-                        waits = 0;
-                        break;
+                        __nanosleep(32);
                     }
-                    if (W == 1) {
-                        // rows of one lane publish inside the loop: leave it only
-                        // when every lane is done or one needs its next chunk
-                        const unsigned w = __reduce_or_sync(
-                            FULL, lane_done ? 0u : (pend != 0 ? 1u : 2u));
-                        if ((w & 2u) || !(w & 1u)) break;
-                    } else if (__any_sync(FULL, pend != before)) {
-                        break;  // something arrived
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (Marker<T>::pending(v[e])) v[e] = look(c[e]);
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    if (!(slots & (1u << e))) continue;
+                    if (act) r.sum = fma(-a[e], v[e], r.sum);  // no entry: adds -0 * 0
+                }
+                if (!more) break;
+                q0 += W * E;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (act) {
+                        c[e] = c2[e];
+                        a[e] = a2[e];
+                        v[e] = T(0);
+                        if (c[e] >= 0) v[e] = look(c[e]);
                     }
-                    if (waits >= p.spin.hot) {
-                        __nanosleep(ns);
-                        ns = ns < p.spin.max_ns ? ns * 2 : p.spin.max_ns;
-                    }
-                } while (true);
-            } else {
-                waits = 0;
-                ns = 32;
             }
+            if (!ok) break;
+            const T tot = group_sum_span<W>(r.sum, FULL, span);
+            if (act && sl == 0 && r.i != p.withhold) {
+                const T val = publishable(tot);
+                if (SMALL)
+                    *(volatile T*)(xpub + own) = val;
+                else
+                    st_relaxed(xpub + own, val);
+                if (p.xacc)
+                    accumulate_with(p, r.i, 0, val, r.xbase);
+                else if (PERM || SMALL)
+                    x[(long long)r.i * p.ldx] = val;
+            }
+            if (W == 32) break;
+            todo = todo && !act;
+            if (!__any_sync(FULL, todo)) break;
+            // lanes of the next level: q0 is still their first chunk's
+            if (todo) q0 = r.beg + sl;
         }
+        if (!ok) tn = stuck_rows<T, W, MAP, PERM, SMALL>(p, t, tn, ticket, xs);
+        if (SMALL && lane == 0) tn = atomicAdd(ticket, 1);
         t = __shfl_sync(FULL, tn, 0);
     }
 }
 
-template <typename T, int W>
-static cudaError_t self_w(const SolveParams& p, int grid, int block, cudaStream_t s) {
-    if (p.xp)  // level-ordered copy: values already gathered, no map
-        self_solve_k1<T, W, false, true><<<grid, block, 0, s>>>(p);
-    else if (p.vmap)
-        self_solve_k1<T, W, true, false><<<grid, block, 0, s>>>(p);
-    else
-        self_solve_k1<T, W, false, false><<<grid, block, 0, s>>>(p);
-    return cudaGetLastError();
+namespace {
+
+// Calls f(kernel) with the instance a launch with these choices uses.
+template <typename T, int W, typename F>
+cudaError_t self_w(bool map, bool perm, bool small, F f) {
+    if (small)
+        return perm ? f(self_solve_k1<T, W, false, true, true>)
+                    : map ? f(self_solve_k1<T, W, true, false, true>)
+                          : f(self_solve_k1<T, W, false, false, true>);
+    return perm ? f(self_solve_k1<T, W, false, true, false>)
+                : map ? f(self_solve_k1<T, W, true, false, false>)
+                      : f(self_solve_k1<T, W, false, false, false>);
 }
 
-template <typename T>
-static cudaError_t self_t(int lanes, const SolveParams& p, int grid, int block, cudaStream_t s) {
+template <typename T, typename F>
+cudaError_t self_t(int lanes, bool map, bool perm, bool small, F f) {
     switch (lanes) {
-        case 1: return self_w<T, 1>(p, grid, block, s);
-        case 2: return self_w<T, 2>(p, grid, block, s);
-        case 4: return self_w<T, 4>(p, grid, block, s);
-        case 8: return self_w<T, 8>(p, grid, block, s);
-        case 16: return self_w<T, 16>(p, grid, block, s);
-        case 32: return self_w<T, 32>(p, grid, block, s);
+        case 1: return self_w<T, 1>(map, perm, small, f);
+        case 2: return self_w<T, 2>(map, perm, small, f);
+        case 4: return self_w<T, 4>(map, perm, small, f);
+        case 8: return self_w<T, 8>(map, perm, small, f);
+        case 16: return self_w<T, 16>(map, perm, small, f);
+        case 32: return self_w<T, 32>(map, perm, small, f);
         default: return cudaErrorInvalidValue;
     }
 }
 
+template <typename F>
+cudaError_t self_any(bool f64, int lanes, bool map, bool perm, bool small, F f) {
+    return f64 ? self_t<double>(lanes, map, perm, small, f)
+               : self_t<float>(lanes, map, perm, small, f);
+}
+
+}  // namespace
+
 cudaError_t launch_self_k1(bool f64, int lanes, const SolveParams& p, int grid, int block,
                            cudaStream_t s) {
-    return f64 ? self_t<double>(lanes, p, grid, block, s) : self_t<float>(lanes, p, grid, block, s);
-}
-
-template <typename T, bool MAP>
-static int occ_k1(int lanes, int block) {
-    int nb = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-    switch (lanes) {
-        case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 1, MAP, false>, block, 0); break;
-        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 2, MAP, false>, block, 0); break;
-        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 4, MAP, false>, block, 0); break;
-        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 8, MAP, false>, block, 0); break;
-        case 16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 16, MAP, false>, block, 0); break;
-        case 32: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, 32, MAP, false>, block, 0); break;
+    if (block > kMaxSelfBlock) {  // the same warps in blocks of kMaxSelfBlock threads
+        grid = (int)(((long long)grid * block + kMaxSelfBlock - 1) / kMaxSelfBlock);
+        block = kMaxSelfBlock;
     }
-    return (e == cudaSuccess && nb > 0) ? nb : 1;
+    // a level-ordered copy holds its values gathered: no map
+    return self_any(f64, lanes, !p.xp && p.vmap, p.xp != nullptr, false, [&](auto k) {
+        k<<<grid, block, 0, s>>>(p);
+        return cudaGetLastError();
+    });
 }
 
-template <typename T>
-static int occ_perm(int lanes, int block) {
+cudaError_t launch_self_small(bool f64, int lanes, const SolveParams& p, int block,
+                              cudaStream_t s) {
+    const size_t smem = (f64 ? 8 : 4) * (size_t)p.n;  // checked by the caller
+    if (block > kMaxSelfBlock) block = kMaxSelfBlock;
+    return self_any(f64, lanes, !p.xp && p.vmap, p.xp != nullptr, true, [&](auto k) {
+        if (smem > 48 * 1024 - 256) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        k<<<1, block, smem, s>>>(p);
+        return cudaGetLastError();
+    });
+}
+
+int self_k1_blocks_per_sm(bool f64, int lanes, bool map, bool perm, int block) {
     int nb = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-#define SPTRSV_OCC(WW) \
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, self_solve_k1<T, WW, false, true>, block, 0)
-    switch (lanes) {
-        case 1: SPTRSV_OCC(1); break;
-        case 2: SPTRSV_OCC(2); break;
-        case 4: SPTRSV_OCC(4); break;
-        case 8: SPTRSV_OCC(8); break;
-        case 16: SPTRSV_OCC(16); break;
-        case 32: SPTRSV_OCC(32); break;
-    }
-#undef SPTRSV_OCC
-    return (e == cudaSuccess && nb > 0) ? nb : 1;
-}
-
-int self_perm_blocks_per_sm(bool f64, int lanes, int block) {
-    return f64 ? occ_perm<double>(lanes, block) : occ_perm<float>(lanes, block);
-}
-
-int self_k1_blocks_per_sm(bool f64, int lanes, bool map, int block) {
-    if (f64) return map ? occ_k1<double, true>(lanes, block) : occ_k1<double, false>(lanes, block);
-    return map ? occ_k1<float, true>(lanes, block) : occ_k1<float, false>(lanes, block);
+    const int run = block > kMaxSelfBlock ? kMaxSelfBlock : block;
+    const cudaError_t e = self_any(f64, lanes, map, perm, false, [&](auto k) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, run, 0);
+    });
+    if (e != cudaSuccess || nb < 1) return 1;
+    nb = (int)((long long)nb * run / block);  // in blocks of the size asked for
+    return nb > 0 ? nb : 1;
 }
 
 }  // namespace sptrsv
