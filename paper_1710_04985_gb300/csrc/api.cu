@@ -160,14 +160,25 @@ int default_lanes(int n, int nnz) {
 }
 
 // Default sub-warp width of the multi-RHS kernels: one lane per column up to
-// 16 lanes, beyond that several columns per lane.  A narrower group holds
-// more rows per warp, so more rows wait ahead of the dependency frontier
-// (128^3 L factor, k = 32: 1.24 ms with 16 lanes against 1.98 ms with 32).
-int mrhs_lanes(int nrhs) {
+// 16 lanes, beyond that several columns per lane; 8 lanes where a level holds
+// enough rows to keep every warp busy anyway.  A narrower group holds more rows
+// per warp, so more rows wait ahead of the dependency frontier, and a row's later
+// columns start while its first ones are still on their way (k = 32 on the
+// 128^3 L factor, 5490 rows per level, 16 / 8 / 4 lanes: 1175 / 1108 / 1377 us;
+// k = 18 on a 27-point grid of 981 rows per level: 2247 / 2456 / 3015 us).
+int mrhs_lanes(int nrhs, double rows_per_level, bool alike) {
     int w = pow2_at_least(nrhs);
     if (w < 4) w = 4;
-    return w > 16 ? 16 : w;
+    const int most = alike && rows_per_level >= 2048 ? 8 : 16;
+    return w > most ? most : w;
 }
+
+// Levels of this many tickets (32 / lanes rows each) and more run the multi-RHS
+// kernel with all the blocks that fit instead of two per SM, unless the caller
+// has set a grid (k = 32 on the 128^3 L factor: 1290 -> 1108 us at 1372 tickets
+// per level; k = 24 on 97 x 101 x 89: 482 -> 435 us at 765; k = 18 on a 27-point
+// grid 1711 -> 1633 us at 490; a 9-point grid of 17 tickets 1294 -> 1413 us).
+constexpr double kMrhsWide = 256.0;
 
 bool capturing(cudaStream_t s) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -221,6 +232,7 @@ struct sptrsv_plan_s {
     unsigned long long* rf_norms = nullptr;  // [0, S) max|r^m|, [S, 2S) max|x^m|
     double anorm = -1.0;                     // ||A||_inf of the current values (-1: unknown)
     int lanes = 4, block = 256, max_blocks = 0;
+    bool shape_set = false;  // by sptrsv_set_tuning
     // per-algorithm single-RHS shapes (lanes 0: use the plan's shape)
     int alg_lanes[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     int alg_block[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -1137,15 +1149,20 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
                           bool acc_first = false) {
     const bool mrhs = nrhs > 1;
     const bool f32_of_f64 = !f64 && P->f64;
+    const Levels& Lt = trans ? P->trn : P->fwd;
+    const double per_level = (double)P->n / (Lt.nlev > 0 ? Lt.nlev : 1);
     // multi-RHS solves have a launch shape of their own (sptrsv_set_mrhs_tuning);
     // a single-RHS solve takes its algorithm's shape if one was set
     const int a = (int)algo;
     const bool own = !mrhs && a >= 0 && a < 8 && P->alg_lanes[a] > 0;
-    const int lanes = mrhs ? (P->mrhs_lanes ? P->mrhs_lanes : mrhs_lanes(nrhs))
+    const int lanes = mrhs ? (P->mrhs_lanes ? P->mrhs_lanes
+                                            : mrhs_lanes(nrhs, per_level, rows_alike(P, Lt, 8)))
                            : (own ? P->alg_lanes[a] : P->lanes);
     const int block = mrhs ? (P->mrhs_block ? P->mrhs_block : P->block)
                            : (own ? P->alg_block[a] : P->block);
-    const int max_blocks = mrhs ? (P->mrhs_max_blocks >= 0 ? P->mrhs_max_blocks : P->max_blocks)
+    const bool wide = mrhs && !P->shape_set && per_level * lanes >= 32.0 * kMrhsWide;
+    const int max_blocks = mrhs ? (P->mrhs_max_blocks >= 0 ? P->mrhs_max_blocks
+                                   : wide ? 0 : P->max_blocks)
                                 : (own ? P->alg_max_blocks[a] : P->max_blocks);
     if (algo == SPTRSV_ALGO_SELF_CHAINS && !mrhs) ST(build_chain(P, trans, lanes, s));
     // The copies hold the plan's element type, and FP32 values beside them
@@ -1193,6 +1210,9 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     p.jlev = L.jlev;
     p.lev = L.lev;
     p.rows_alike = rows_alike(P, L, lanes) ? 1 : 0;
+    // a unit diagonal need not be stored: then max_len counts no diagonal
+    const MrhsRows mrows = !p.rows_alike ? kMrhsApart
+                           : L.max_len - (P->unit ? 0 : 1) <= kChunk ? kMrhsShort : kMrhsAlike;
     p.b = b;
     p.ldb = ldb;
     p.x = x;
@@ -1213,7 +1233,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         for (int m = 0; m < L.nlev; ++m) {
             p.kbeg = L.h_ilev[m];
             p.cnt = L.h_ilev[m + 1] - L.h_ilev[m];
-            CK(mrhs ? launch_mrhs(f64, lanes, false, p, 0, block, s)
+            CK(mrhs ? launch_mrhs(f64, lanes, false, kMrhsApart, p, 0, block, s)
                     : launch_level_k1(f64, lanes, p, block, s));
         }
         ST(prof_end(P, s));
@@ -1291,12 +1311,12 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         const int R = 32 / lanes;
         const long long tickets = ((long long)P->n + R - 1) / R;
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
-        long long grid = (long long)self_blocks_per_sm(f64, lanes, true, false, block) * P->num_sms;
+        long long grid = (long long)mrhs_blocks_per_sm(f64, lanes, false, true, mrows, block) * P->num_sms;
         if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
         if (grid > want_blocks) grid = want_blocks;
         if (grid < 1) grid = 1;
         ST(prof_begin(P, s));
-        CK(launch_mrhs(f64, lanes, true, p, (int)grid, block, s));
+        CK(launch_mrhs(f64, lanes, true, mrows, p, (int)grid, block, s));
         ST(prof_end(P, s));
         launches = 2;
     } else if (permuted) {
@@ -1360,8 +1380,9 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         const int R = 32 / lanes;
         const long long tickets = ((long long)P->n + R - 1) / R;
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
-        long long grid =
-            (long long)self_blocks_per_sm(f64, lanes, mrhs, trans, block) * P->num_sms;
+        long long grid = P->num_sms *
+                         (long long)(mrhs ? mrhs_blocks_per_sm(f64, lanes, trans, false, mrows, block)
+                                          : self_k1_blocks_per_sm(f64, lanes, trans, false, block));
         if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
         if (grid > want_blocks) grid = want_blocks;
         if (grid < 1) grid = 1;
@@ -1386,7 +1407,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             ST(prof_end(P, s));
         } else {
             ST(prof_begin(P, s));
-            CK(mrhs ? launch_mrhs(f64, lanes, true, p, (int)grid, block, s)
+            CK(mrhs ? launch_mrhs(f64, lanes, true, mrows, p, (int)grid, block, s)
                     : launch_self_k1(f64, lanes, p, (int)grid, block, s));
             ST(prof_end(P, s));
         }
@@ -1900,6 +1921,7 @@ sptrsv_status_t sptrsv_set_tuning(sptrsv_plan_t plan, int lanes_per_row, int blo
     plan->lanes = w;
     plan->block = block_size;
     plan->max_blocks = max_blocks;
+    plan->shape_set = true;
     for (int a = 0; a < 8; ++a) plan->alg_lanes[a] = 0;
     return SPTRSV_OK;
 }

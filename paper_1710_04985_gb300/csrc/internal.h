@@ -94,10 +94,14 @@ cudaError_t launch_prep_self(bool f64, int n, int nrhs, void* x, long long ldx, 
 cudaError_t launch_self_k1(bool f64, int lanes, const SolveParams& p, int grid, int block,
                            cudaStream_t s);
 cudaError_t launch_level_k1(bool f64, int lanes, const SolveParams& p, int block, cudaStream_t s);
-cudaError_t launch_mrhs(bool f64, int lanes, bool self, const SolveParams& p, int grid, int block,
-                        cudaStream_t s);
+// How the self-scheduled multi-RHS kernel takes a ticket's rows: every row at its
+// own pace, or as one (rows alike), with rows of one chunk (kChunk entries beside
+// the diagonal) only or of any length.
+enum MrhsRows { kMrhsApart, kMrhsAlike, kMrhsShort };
+cudaError_t launch_mrhs(bool f64, int lanes, bool self, MrhsRows rows, const SolveParams& p,
+                        int grid, int block, cudaStream_t s);
 // Resident blocks per SM of the kernel a launch with these choices would use.
-int self_blocks_per_sm(bool f64, int lanes, bool mrhs, bool map, int block);
+int mrhs_blocks_per_sm(bool f64, int lanes, bool map, bool perm, MrhsRows rows, int block);
 // Tiled self-scheduled solve (solve_tiled.cu): tiles of `tile_rows`
 // consecutive positions of the substitution order (p.ipos == nullptr) or of
 // the level order jlev (p.ipos != nullptr); tile_rows * sizeof(T) <= 48 KB.
