@@ -327,28 +327,30 @@ sptrsv_status_t kahn_levels(sptrsv_plan_t P, const int* ptr, const int* idx, con
                             cudaStream_t s) {
     const int n = P->n;
     int* scratch = nullptr;
-    // Layout (ints): [0, 2) the 64-bit barrier counter, which must be 8-byte
-    // aligned and so comes first (cudaMalloc returns 256-byte aligned
-    // memory); [2, 6) the queue end / rotating level counters (the roots are
-    // counted in [2]; [5] = rows leveled by the persistent form); [6] level
-    // count; [7, 10) the persistent form's narrow-run state; [10, 12) pad;
-    // then count0, count, queue.
-    CK(cudaMalloc(&scratch, sizeof(int) * (3 * (size_t)n + 12)));
-    unsigned long long* arrivals = (unsigned long long*)scratch;
-    int* qend = scratch + 2;
-    int* nlev_dev = scratch + 6;
-    int* ctl = scratch + 7;
-    int* count0 = scratch + 12;
+    // Layout (ints): [0, 6) the three 64-bit barrier words and, from 16, the
+    // edge ranges of the persistent form (int2 each), which must be 8-byte
+    // aligned and so come first (cudaMalloc returns 256-byte aligned memory);
+    // [6, 10) the queue end / rotating level counters (the roots are counted
+    // in [6]; [9] = rows leveled by the persistent form); [10] level count;
+    // [11, 14) the persistent form's narrow-run state; then count0, count, queue.
+    CK(cudaMalloc(&scratch, sizeof(int) * (5 * (size_t)n + 16)));
+    unsigned long long* words = (unsigned long long*)scratch;
+    int* qend = scratch + 6;
+    int* nlev_dev = scratch + 10;
+    int* ctl = scratch + 11;
+    int2* span = (int2*)(scratch + 16);
+    int* count0 = scratch + 16 + 2 * (size_t)n;
     int* count = count0 + n;
     int* queue = count + n;
-    cudaError_t e = cudaMemsetAsync(scratch, 0, 12 * sizeof(int), s);
+    cudaError_t e = cudaMemsetAsync(scratch, 0, 16 * sizeof(int), s);
     if (e == cudaSuccess) e = launch_column_counts(n, ptr, idx, count0, s);
     if (e == cudaSuccess) e = launch_kahn_roots(n, count0, count, L.lev, queue, qend, s);
     int h_last = 0, level = 0;
     if (e == cudaSuccess && persistent) {
         // One block of 1024 threads per SM keeps the grid barrier short (one
-        // arrival per SM); a level with at most one row per warp of a block
-        // runs on block 0 alone.
+        // arrival per SM); a lane per edge of an average row; a level that one
+        // block takes at once runs on block 0 alone.
+        const int klanes = pow2_at_least((double)P->nnz / (n > 0 ? n : 1));
         int block = (int)env_ll("SPTRSV_KAHN_BLOCK", 1024);
         if (block < 64 || block > 1024 || block % 32 != 0) block = 1024;
         long long per_sm = env_ll("SPTRSV_KAHN_BLOCKS_PER_SM", 1);
@@ -356,15 +358,15 @@ sptrsv_status_t kahn_levels(sptrsv_plan_t P, const int* ptr, const int* idx, con
         if (per_sm > fit) per_sm = fit;
         long long grid = per_sm * P->num_sms;
         if (grid < 1) grid = 1;
-        const int narrow = (int)env_ll("SPTRSV_KAHN_NARROW", block / 32);
+        const int narrow = (int)env_ll("SPTRSV_KAHN_NARROW", block / klanes);
         // Probe (automatic method only): after 256 levels, fewer than 112
         // rows per level on average means a deep, narrow graph, where a
         // grid barrier per level loses to the sweep (measured: 2.2-3.6 us
         // per level against the sweep's 1.2-1.3 us on such graphs); levels
         // still widening at that point are judged again at level 1024.
         const int probe_level = probe ? 256 : 0;
-        e = launch_kahn_persistent(dptr, didx, count, L.lev, queue, qend, ctl, n, narrow,
-                                   probe_level, 112, arrivals, nlev_dev, P->status,
+        e = launch_kahn_persistent(dptr, didx, count, L.lev, queue, span, qend, ctl, n, narrow,
+                                   klanes, probe_level, 112, words, nlev_dev, P->status,
                                    P->spin.limit, (int)grid, block, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&level, nlev_dev, sizeof(int),
                                                   cudaMemcpyDeviceToHost, s);

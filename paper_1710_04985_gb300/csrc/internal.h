@@ -298,16 +298,18 @@ cudaError_t launch_kahn_level(const int* dptr, const int* didx, int* count, int*
                               unsigned long long* status, int max_grid, cudaStream_t s);
 int kahn_persistent_blocks_per_sm(int block);
 // cnt[0] = roots queued by launch_kahn_roots, cnt[1] = cnt[2] = 0; on exit
-// cnt[3] = rows leveled and *nlev_out = levels.  ctl: 3 ints of scratch.
+// cnt[3] = rows leveled and *nlev_out = levels.  ctl: 3 ints, span: n int2 of
+// scratch; words: three zeros.
+// `lanes` lanes (a power of two up to 32) remove a row's outgoing edges.
 // Levels of at most `narrow` rows run on block 0 alone.  With probe_level
 // > 0, the launch gives up (*nlev_out = -1) when fewer than
 // level * probe_min_avg rows are leveled after probe_level levels, unless
 // the levels are still widening, in which case it looks again (once) at
 // four times that level with a 1.5 times larger average.
 cudaError_t launch_kahn_persistent(const int* dptr, const int* didx, int* count, int* lev,
-                                   int* queue, int* cnt, int* ctl, int n, int narrow,
-                                   int probe_level, int probe_min_avg,
-                                   unsigned long long* arrivals, int* nlev_out,
+                                   int* queue, int2* span, int* cnt, int* ctl, int n, int narrow,
+                                   int lanes, int probe_level, int probe_min_avg,
+                                   unsigned long long* words, int* nlev_out,
                                    unsigned long long* status, long long limit, int grid,
                                    int block, cudaStream_t s);
 

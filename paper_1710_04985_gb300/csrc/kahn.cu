@@ -94,26 +94,28 @@ cudaError_t launch_kahn_level(const int* dptr, const int* didx, int* count, int*
     return cudaGetLastError();
 }
 
-// Grid-wide barrier for a cooperative launch: every block adds one arrival
-// per barrier to a 64-bit counter (zero at launch) and waits until the
-// counter reaches blocks * generation.  Release/acquire order the frontier
-// writes of one generation before the reads of the next.  Returns false if
-// the wait ran past the limit (then SPTRSV_ERR_TIMEOUT is recorded).
-__device__ __forceinline__ bool grid_barrier(unsigned long long* arrivals,
-                                             unsigned long long target, long long limit,
+// Grid-wide barrier number `gen` of a cooperative launch: every block adds one
+// arrival, and `add` to a total, to one of three 64-bit words used in turn (zero
+// at launch) and waits until all have arrived; *total is the sum of their `add`.
+// A barrier's word is cleared after the next barrier (every block has left it by
+// then) and used again by the one after that.  Release/acquire order the writes
+// of one generation before the reads of the next.  Returns false if the wait ran
+// past the limit (then SPTRSV_ERR_TIMEOUT is recorded).
+__device__ __forceinline__ bool grid_barrier(unsigned long long* words, unsigned gen, int add,
+                                             int* total, long long limit,
                                              unsigned long long* status, int row) {
-    __shared__ int s_ok;
+    __shared__ int s_ok, s_total;
     __syncthreads();
     if (threadIdx.x == 0) {
+        unsigned long long* w = words + gen % 3;
+        const unsigned long long mine = ((unsigned long long)(unsigned)add << 32) | 1ull;
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(mine) : "memory");
         int ok = 1;
-        __threadfence();
-        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrivals) : "memory");
         long long spins = 0;
+        unsigned long long v;
         while (true) {
-            unsigned long long v;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(arrivals)
-                         : "memory");
-            if (v >= target) break;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(w) : "memory");
+            if ((unsigned)v >= gridDim.x) break;
             if (++spins >= limit) {
                 report(status, row, kCodeTimeout);
                 ok = 0;
@@ -121,83 +123,99 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* arrivals,
             }
             if (spins > 64) __nanosleep(64);
         }
+        if (blockIdx.x == 0) *(volatile unsigned long long*)(words + (gen + 2) % 3) = 0;
         s_ok = ok;
+        s_total = (int)(v >> 32);
     }
     __syncthreads();
+    *total = s_total;
     return s_ok != 0;
 }
 
-// Removes the frontier queue[base, base + size) of level `level` with the
-// warps [w0, w0 + nw): a warp per frontier row, its lanes over the row's
-// outgoing edges; roots of level + 1 are counted in *tail and stored after
-// the frontier.  Queue entries may have been written by other SMs: they are
-// read from L2 (__ldcg), never from a stale L1 line.
-__device__ __forceinline__ void kahn_frontier(const int* __restrict__ dptr,
-                                              const int* __restrict__ didx, int* count, int* lev,
-                                              int* queue, int* tail, int n, long long base,
-                                              int size, int level, long long w0, long long nw,
-                                              int lane, unsigned long long* status) {
-    int* next = queue + base + size;
-    for (long long w = w0; w < size; w += nw) {
-        const int i = __ldcg(queue + base + w);
-        const int beg = dptr[i], end = dptr[i + 1];
-        for (int q = beg + lane; q < end; q += 32) {
-            const int r = didx[q];
-            if (r == i) continue;
-            if (atomicSub(count + r, 1) == 1) {
-                lev[r] = level + 1;
-                const int at = atomicAdd(tail, 1);
-                if (base + size + at < n) next[at] = r;
-                else report(status, r, kCodeInternal);
-            }
+// Roots a block gathers in shared memory.
+constexpr int kGather = 2048;
+struct Gather {
+    int row[kGather], beg[kGather], end[kGather];
+    int cnt;
+    int at;
+};
+
+// Persistent driver.  The frontier of level L is queue[base_L, base_L +
+// size_L), with the rows' outgoing edges [beg, end) in span; its removal appends
+// the roots of level L + 1 right after it.  The places of a level's roots are
+// counted in three rotating words cnt[L % 3]: the roots of level L + 1 in
+// cnt[(L + 1) % 3], while block 0 clears cnt[(L + 2) % 3], which nobody adds to
+// before the next barrier.  The number of roots itself comes with the barrier.
+//
+// What bounds a level is the chain root -> edge -> counter of the dependent ->
+// place in the queue -> barrier, an L2 latency each, so as many rows as possible
+// go through it at once (`lanes` lanes to a row: a lane per edge of an average
+// row; consecutive warps of the frontier on different SMs), a root's edge range
+// is loaded by the block that found it while its place is on the way, and a
+// block gathers its roots in shared memory and takes their places with one
+// atomic (one atomic per root on the one counter of a level, 5490 roots on the
+// 128^3 factor, had all of them queue up in L2).  Plan setup of the 128^3 ILU(0)
+// L factor 4.26 -> 3.42 ms, of the 9-point 1012 x 974 lower triangle (narrow
+// levels) 13.7 -> 10.9 ms, of the 27-point 70 x 89 x 103 one 4.77 -> 4.24 ms.
+//
+// Wide levels run on the whole grid, one grid barrier each.  A level of at
+// most `narrow` rows runs on block 0 alone, which keeps going through
+// consecutive narrow levels with the frontier in shared memory and block
+// barriers only, and then publishes the frontier and (base, size, level) in
+// ctl[0..2]; the other blocks meanwhile wait at the grid barrier that closes the
+// run.  A run opens with one more grid barrier, after which every block has
+// read the size it starts from.  cnt[0] holds the roots queued by kahn_roots_k;
+// cnt[1], cnt[2] and words[0..2] start at zero.  Writes the level count and
+// cnt[3] = rows leveled.
+constexpr int kNarrowRun = 4096;
+
+// Removes row i's edges [beg, end) with the lanes sl, sl + lanes, ...; new roots
+// go to g, those beyond its room to over(place, root), place >= kGather.
+template <typename F>
+__device__ __forceinline__ void kahn_remove_row(const int* __restrict__ didx, int* count, int* lev,
+                                                int level, int i, int beg, int end, int sl,
+                                                int lanes, Gather& g, F over) {
+    for (int q = beg + sl; q < end; q += lanes) {
+        const int r = didx[q];
+        if (r == i) continue;
+        if (atomicSub(count + r, 1) == 1) {
+            lev[r] = level + 1;
+            const int at = atomicAdd(&g.cnt, 1);
+            if (at < kGather) g.row[at] = r;
+            else over(at, r);
         }
     }
 }
 
-// Persistent driver.  The frontier of level L is queue[base_L, base_L +
-// size_L); its removal appends the roots of level L + 1 right after it.
-// Level sizes live in three rotating counters cnt[L % 3]: the value read
-// after a barrier must not move while slower readers still read it, so the
-// roots of level L + 1 are counted in cnt[(L+1) % 3] (not in the one being
-// read), and block 0 clears cnt[(L+2) % 3] at the start of level L: every
-// reader read that counter (size of level L - 1) before the barrier that
-// opened level L, and nobody appends to it before the next one.
-//
-// Wide levels run on the whole grid, one grid barrier each.  A level of at
-// most `narrow` rows runs on block 0 alone, which keeps going through
-// consecutive narrow levels separated only by block barriers (no grid-wide
-// step) and then publishes (base, size, level) in ctl[0..2]; the other
-// blocks meanwhile wait at the grid barrier that closes the run.  A run
-// opens with one more grid barrier, after which every block has read the
-// size it starts from, so block 0 may clear and reuse that counter.  Deep,
-// narrow dependency graphs thus cost a block barrier per level, not a grid
-// barrier.  cnt[0] holds the roots queued by kahn_roots_k; cnt[1], cnt[2]
-// start at zero.  Writes the level count and cnt[3] = rows leveled.
-constexpr int kNarrowRun = 4096;
-
-__global__ void kahn_persistent_k(const int* __restrict__ dptr, const int* __restrict__ didx,
-                                  int* count, int* lev, int* queue, int* cnt, int* ctl, int n,
-                                  int narrow, int probe_level, int probe_min_avg,
-                                  unsigned long long* arrivals, int* nlev_out,
-                                  unsigned long long* status, long long limit) {
+__global__ void __launch_bounds__(1024)
+    kahn_persistent_k(const int* __restrict__ dptr, const int* __restrict__ didx, int* count,
+                      int* lev, int* queue, int2* span, int* cnt, int* ctl, int n, int narrow,
+                      int lanes, int probe_level, int probe_min_avg, unsigned long long* words,
+                      int* nlev_out, unsigned long long* status, long long limit) {
+    extern __shared__ __align__(16) unsigned char kahn_smem[];
+    Gather* const g = (Gather*)kahn_smem;  // two of them
     const int lane = threadIdx.x & 31;
-    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long wid = (((long long)blockIdx.x * blockDim.x) >> 5) + (threadIdx.x >> 5);
+    const int per = 32 / lanes, sl = lane % lanes;
     const int bwarps = blockDim.x >> 5, bwid = threadIdx.x >> 5;
-    unsigned long long gen = 0;
+    const long long warps = (long long)gridDim.x * bwarps;
+    const long long wid = (long long)bwid * gridDim.x + blockIdx.x;
+    unsigned gen = 0;
     long long base = 0;
     int size = *(volatile int*)cnt;  // roots, queued before this launch
-    int level = 0;
+    int level = 0, total = 0;
+    bool spans = false;  // the frontier's edge ranges are in span (not level 0's)
     // Level at which the next probe is taken (0: none left).
     int next_probe = probe_level > 0 ? probe_level : 0;
     bool postponed = false;
+    if (threadIdx.x == 0) g[0].cnt = g[1].cnt = 0;
+    __syncthreads();
     while (size > 0) {
-        // Early exit for deep, narrow graphs (a grid barrier per level costs
-        // more there than the sweep): every block sees the same (base, size,
-        // level) here, so all of them decide alike.  Levels that are still
-        // widening (the current one at least 1.5 times the average so far)
-        // get one second look at four times the level, which then asks for
-        // a 1.5 times larger average.
+        // Early exit for deep, narrow graphs (a level costs more here than in
+        // the sweep): every block sees the same (base, size, level) here, so
+        // all of them decide alike.  Levels that are still widening (the
+        // current one at least 1.5 times the average so far) get one second
+        // look at four times the level, which then asks for a 1.5 times larger
+        // average.
         if (next_probe > 0 && level >= next_probe) {
             next_probe = 0;
             const long long need = postponed ? (3ll * probe_min_avg) / 2 : probe_min_avg;
@@ -211,41 +229,72 @@ __global__ void kahn_persistent_k(const int* __restrict__ dptr, const int* __res
                 }
             }
         }
-        if (size <= narrow) {
-            // Every block must have read `size` (the counter of the grid
-            // barrier just passed) before block 0 runs ahead: its next levels
-            // clear and reuse that counter.  One extra grid barrier per run.
-            ++gen;
-            if (!grid_barrier(arrivals, gen * gridDim.x, limit, status, level)) return;
+        if (size <= narrow && size <= kGather) {
+            // Every block must have read the state of the barrier just passed
+            // before block 0 runs ahead.  One extra grid barrier per run.
+            if (!grid_barrier(words, gen++, 0, &total, limit, status, level)) return;
             if (blockIdx.x == 0) {
+                int cur = 0;
+                for (int k = threadIdx.x; k < size; k += blockDim.x) {
+                    const int r = __ldcg(queue + base + k);
+                    g[0].row[k] = r;
+                    g[0].beg[k] = dptr[r];
+                    g[0].end[k] = dptr[r + 1];
+                }
+                __syncthreads();
                 // at most kNarrowRun levels per run, so the other blocks' wait
                 // at the closing barrier stays far below its spin limit; a run
                 // also stops at the probe level so that the probe is taken
-                for (int run = 0; run < kNarrowRun && size > 0 && size <= narrow &&
-                                   (next_probe == 0 || level < next_probe);
-                     ++run) {
-                    if (threadIdx.x == 0) cnt[(level + 2) % 3] = 0;
+                int run = 0;
+                do {
+                    Gather& to = g[cur ^ 1];
+                    int* next = queue + base + size;
+                    const long long room = (long long)n - base - size;
+                    for (int f = bwid * per + lane / lanes; f < size; f += bwarps * per)
+                        kahn_remove_row(didx, count, lev, level, g[cur].row[f], g[cur].beg[f],
+                                        g[cur].end[f], sl, lanes, to, [&](int at, int r) {
+                                            if (at < room) next[at] = r;
+                                            else report(status, r, kCodeInternal);
+                                        });
                     __syncthreads();
-                    int* tail = cnt + (level + 1) % 3;
-                    kahn_frontier(dptr, didx, count, lev, queue, tail, n, base, size, level, bwid,
-                                  bwarps, lane, status);
-                    __syncthreads();  // every append of this level has been performed
-                    int nsz;
-                    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(nsz) : "l"(tail)
-                                 : "memory");
-                    __syncthreads();  // read by all before the next level appends
+                    const int found = to.cnt;
+                    const int kept = found < kGather ? found : kGather;
+                    for (int k = threadIdx.x; k < kept; k += blockDim.x) {
+                        const int r = to.row[k];
+                        to.beg[k] = dptr[r];
+                        to.end[k] = dptr[r + 1];
+                    }
+                    __syncthreads();
+                    if (threadIdx.x == 0) to.cnt = 0;
                     base += size;
-                    size = nsz;
+                    size = found;
                     ++level;
+                    ++run;
+                    cur ^= 1;
+                } while (run < kNarrowRun && size > 0 && size <= narrow && size <= kGather &&
+                         (next_probe == 0 || level < next_probe));
+                // the frontier for the grid
+                for (int k = threadIdx.x; k < size; k += blockDim.x) {
+                    if (base + k >= n) {
+                        report(status, (int)base, kCodeInternal);
+                        break;
+                    }
+                    if (k < kGather) {
+                        queue[base + k] = g[cur].row[k];
+                        span[base + k] = make_int2(g[cur].beg[k], g[cur].end[k]);
+                    } else {
+                        const int r = __ldcg(queue + base + k);
+                        span[base + k] = make_int2(dptr[r], dptr[r + 1]);
+                    }
                 }
                 if (threadIdx.x == 0) {
                     ctl[0] = (int)base;
                     ctl[1] = size;
                     ctl[2] = level;
+                    cnt[0] = cnt[1] = cnt[2] = 0;
                 }
             }
-            ++gen;
-            if (!grid_barrier(arrivals, gen * gridDim.x, limit, status, level)) return;
+            if (!grid_barrier(words, gen++, 0, &total, limit, status, level)) return;
             int st[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k)
@@ -254,19 +303,63 @@ __global__ void kahn_persistent_k(const int* __restrict__ dptr, const int* __res
             base = st[0];
             size = st[1];
             level = st[2];
+            spans = true;
             continue;
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) cnt[(level + 2) % 3] = 0;
         int* tail = cnt + (level + 1) % 3;
-        kahn_frontier(dptr, didx, count, lev, queue, tail, n, base, size, level, wid, warps, lane,
-                      status);
-        ++gen;
-        if (!grid_barrier(arrivals, gen * gridDim.x, limit, status, level)) return;
-        int nsz;
-        asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(nsz) : "l"(tail) : "memory");
+        int* next = queue + base + size;
+        int2* next_span = span + base + size;
+        const long long room = (long long)n - base - size;  // places that are left
+        for (long long w = wid; w * per < size; w += warps) {
+            const long long f = w * per + lane / lanes;
+            if (f >= size) continue;
+            const int i = __ldcg(queue + base + f);
+            int2 s;
+            if (spans) s = __ldcg(span + base + f);
+            else s = make_int2(dptr[i], dptr[i + 1]);
+            kahn_remove_row(didx, count, lev, level, i, s.x, s.y, sl, lanes, g[0],
+                            [&](int, int r) {
+                                const int at = atomicAdd(tail, 1);
+                                if (at < room) {
+                                    next[at] = r;
+                                    next_span[at] = make_int2(dptr[r], dptr[r + 1]);
+                                } else {
+                                    report(status, r, kCodeInternal);
+                                }
+                            });
+        }
+        __syncthreads();
+        const int mine = g[0].cnt < kGather ? g[0].cnt : kGather;
+        const int found = g[0].cnt;  // with the ones queued one by one
+        if (threadIdx.x == 0 && mine > 0) g[0].at = atomicAdd(tail, mine);
+        int beg = 0, end = 0;  // of this thread's first root, while the place comes
+        if ((int)threadIdx.x < mine) {
+            beg = dptr[g[0].row[threadIdx.x]];
+            end = dptr[g[0].row[threadIdx.x] + 1];
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < mine; k += blockDim.x) {
+            const int r = g[0].row[k];
+            if (k != (int)threadIdx.x) {
+                beg = dptr[r];
+                end = dptr[r + 1];
+            }
+            const int at = g[0].at + k;
+            if (at < room) {
+                next[at] = r;
+                next_span[at] = make_int2(beg, end);
+            } else {
+                report(status, r, kCodeInternal);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) g[0].cnt = 0;
+        if (!grid_barrier(words, gen++, found, &total, limit, status, level)) return;
         base += size;
-        size = nsz;
+        size = total;
         ++level;
+        spans = true;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *nlev_out = level;
@@ -274,28 +367,37 @@ __global__ void kahn_persistent_k(const int* __restrict__ dptr, const int* __res
     }
 }
 
+// Shared memory of the kernel: 48 KB and a little, so it is opted in to.
+static cudaError_t kahn_attr() {
+    return cudaFuncSetAttribute(kahn_persistent_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(2 * sizeof(Gather)));
+}
+
 int kahn_persistent_blocks_per_sm(int block) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kahn_persistent_k, block, 0) !=
-            cudaSuccess ||
+    if (kahn_attr() != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kahn_persistent_k, block,
+                                                      2 * sizeof(Gather)) != cudaSuccess ||
         nb < 1)
         return 1;
     return nb;
 }
 
 cudaError_t launch_kahn_persistent(const int* dptr, const int* didx, int* count, int* lev,
-                                   int* queue, int* cnt, int* ctl, int n, int narrow,
-                                   int probe_level, int probe_min_avg,
-                                   unsigned long long* arrivals, int* nlev_out,
+                                   int* queue, int2* span, int* cnt, int* ctl, int n, int narrow,
+                                   int lanes, int probe_level, int probe_min_avg,
+                                   unsigned long long* words, int* nlev_out,
                                    unsigned long long* status, long long limit, int grid,
                                    int block, cudaStream_t s) {
-    void* args[] = {(void*)&dptr,        (void*)&didx,          (void*)&count,
-                    (void*)&lev,         (void*)&queue,         (void*)&cnt,
-                    (void*)&ctl,         (void*)&n,             (void*)&narrow,
-                    (void*)&probe_level, (void*)&probe_min_avg, (void*)&arrivals,
-                    (void*)&nlev_out,    (void*)&status,        (void*)&limit};
+    cudaError_t e = kahn_attr();
+    if (e != cudaSuccess) return e;
+    void* args[] = {(void*)&dptr,   (void*)&didx,        (void*)&count,         (void*)&lev,
+                    (void*)&queue,  (void*)&span,        (void*)&cnt,           (void*)&ctl,
+                    (void*)&n,      (void*)&narrow,      (void*)&lanes,         (void*)&probe_level,
+                    (void*)&probe_min_avg, (void*)&words, (void*)&nlev_out,     (void*)&status,
+                    (void*)&limit};
     return cudaLaunchCooperativeKernel((const void*)kahn_persistent_k, dim3(grid), dim3(block),
-                                       args, 0, s);
+                                       args, 2 * sizeof(Gather), s);
 }
 
 }  // namespace sptrsv
