@@ -471,27 +471,22 @@ __global__ void __launch_bounds__(kScanThreads) scan_chunks_k(const int* __restr
 }
 
 // out[0..m]: exclusive prefix sums of in[0..m-1], out[m] = total (in and
-// out must not overlap).  The block sums take at most kScanBlocks + 1 ints
-// of stream-ordered scratch (setup paths only; never under capture).
-cudaError_t launch_exclusive_scan(const int* in, int* out, int m, cudaStream_t s) {
+// out must not overlap).  sums: kScanSums ints of scratch.
+cudaError_t launch_exclusive_scan(const int* in, int* out, int m, int* sums, cudaStream_t s) {
     if (m <= 0) {
         return cudaMemsetAsync(out, 0, sizeof(int), s);
     }
+    static_assert(kScanBlocks + 1 <= kScanSums, "block sums");
     const long long per_block_min = kScanThreads;
     long long nb = ((long long)m + per_block_min - 1) / per_block_min;
     if (nb > kScanBlocks) nb = kScanBlocks;
     long long chunk = ((long long)m + nb - 1) / nb;
     chunk = (chunk + kScanThreads - 1) / kScanThreads * kScanThreads;
     nb = ((long long)m + chunk - 1) / chunk;
-    int* sums = nullptr;
-    cudaError_t e = cudaMallocAsync(&sums, sizeof(int) * (size_t)(nb + 1), s);
-    if (e != cudaSuccess) return e;
     scan_block_sums_k<<<(int)nb, kScanThreads, 0, s>>>(in, m, chunk, sums);
     scan_sums_k<<<1, kScanThreads, 0, s>>>(sums, (int)nb);
     scan_chunks_k<<<(int)nb, kScanThreads, 0, s>>>(in, out, m, chunk, sums, (int)nb);
-    e = cudaGetLastError();
-    cudaError_t f = cudaFreeAsync(sums, s);
-    return e != cudaSuccess ? e : f;
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ radix sort
@@ -588,7 +583,8 @@ cudaError_t launch_iota(int* out, int m, cudaStream_t s) {
 
 cudaError_t radix_sort_values(const int* keys_in, const int* vals_in, int m, int bits,
                               int* vals_out, int* k_a, int* v_a, int* k_b, int* v_b, int* hist,
-                              int* hist_scan, unsigned long long* status, cudaStream_t s) {
+                              int* hist_scan, int* sums, unsigned long long* status,
+                              cudaStream_t s) {
     if (m == 0) return cudaSuccess;
     const int passes = (bits + 7) / 8;
     if (passes == 0) {
@@ -606,7 +602,7 @@ cudaError_t radix_sort_values(const int* keys_in, const int* vals_in, int m, int
         rs_hist_k<<<nb, kRsThreads, 0, s>>>(kin, m, shift, hist, nb);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = launch_exclusive_scan(hist, hist_scan, 256 * nb, s);
+        e = launch_exclusive_scan(hist, hist_scan, 256 * nb, sums, s);
         if (e != cudaSuccess) return e;
         rs_scatter_k<<<nb, kRsThreads, 0, s>>>(kin, vin, m, shift, hist_scan, nb, kout, vout,
                                                  status);

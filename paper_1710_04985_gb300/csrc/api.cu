@@ -58,6 +58,7 @@ struct Levels {
     int* count0 = nullptr;
     int* count = nullptr;
     int method = SPTRSV_ANALYSIS_SWEEP;  // the analysis that produced these levels
+    bool in_arena = false;               // lev, ilev, jlev, ipos are the plan's arena's
     // Part order (SPTRSV_ALGO_SELF_PARTITIONED, built on first use and again
     // when the part size changes): position k holds row qord[k], rows in parts
     // of qS consecutive rows, by level inside a part; qipos is its inverse and
@@ -218,6 +219,14 @@ struct sptrsv_plan_s {
     int* tmap = nullptr;
     int* counters = nullptr;  // [0] ticket, [1] level count, [2] longest row
     unsigned long long* status = nullptr;
+    int* scan_sums = nullptr;     // kScanSums ints
+    // One allocation for the counters, the status word, the scan's sums, the
+    // transposed pattern and the forward levels; and the scratch of a setup
+    // call, kept until the call returns (ScratchScope).  A cudaMalloc takes
+    // 60-110 us and a cudaFree 45-110 us whatever the size.
+    void* arena = nullptr;
+    void* scratch = nullptr;
+    size_t scratch_bytes = 0;
     void* bcopy = nullptr;
     size_t bcopy_bytes = 0;
     float* vals32 = nullptr;
@@ -259,10 +268,12 @@ struct sptrsv_plan_s {
 namespace {
 
 void free_levels(Levels& L) {
-    cudaFree(L.lev);
-    cudaFree(L.ilev);
-    cudaFree(L.jlev);
-    cudaFree(L.ipos);
+    if (!L.in_arena) {
+        cudaFree(L.lev);
+        cudaFree(L.ilev);
+        cudaFree(L.jlev);
+        cudaFree(L.ipos);
+    }
     for (int* t : L.torder) cudaFree(t);
     cudaFree(L.pptr);
     cudaFree(L.pidx);
@@ -282,11 +293,8 @@ void destroy(sptrsv_plan_t P) {
     DeviceGuard g(P->device);
     free_levels(P->fwd);
     free_levels(P->trn);
-    cudaFree(P->tptr);
-    cudaFree(P->tidx);
-    cudaFree(P->tmap);
-    cudaFree(P->counters);
-    cudaFree(P->status);
+    cudaFree(P->arena);
+    cudaFree(P->scratch);
     cudaFree(P->bcopy);
     cudaFree(P->vals32);
     cudaFree(P->r32);
@@ -297,6 +305,32 @@ void destroy(sptrsv_plan_t P) {
     cudaFree(P->rf_norms);
     for (cudaEvent_t e : P->ev) cudaEventDestroy(e);
     delete P;
+}
+
+// The scratch of a setup call: grown on demand, given back when the call
+// returns.  What it holds is used by kernels of the call's stream only, and
+// every user of it synchronises that stream before the scope ends.
+struct ScratchScope {
+    sptrsv_plan_t P;
+    explicit ScratchScope(sptrsv_plan_t plan) : P(plan) {}
+    ~ScratchScope() {
+        cudaFree(P->scratch);
+        P->scratch = nullptr;
+        P->scratch_bytes = 0;
+    }
+};
+cudaError_t scratch_ints(sptrsv_plan_t P, size_t ints, int** out) {
+    const size_t want = sizeof(int) * (ints > 0 ? ints : 1);
+    if (P->scratch_bytes < want) {
+        cudaFree(P->scratch);  // waits for the kernels that use it
+        P->scratch = nullptr;
+        P->scratch_bytes = 0;
+        const cudaError_t e = cudaMalloc(&P->scratch, want);
+        if (e != cudaSuccess) return e;
+        P->scratch_bytes = want;
+    }
+    *out = (int*)P->scratch;
+    return cudaSuccess;
 }
 
 // Reads and clears the status word (synchronises s).  Returns the code and
@@ -333,7 +367,7 @@ sptrsv_status_t kahn_levels(sptrsv_plan_t P, const int* ptr, const int* idx, con
     // [6, 10) the queue end / rotating level counters (the roots are counted
     // in [6]; [9] = rows leveled by the persistent form); [10] level count;
     // [11, 14) the persistent form's narrow-run state; then count0, count, queue.
-    CK(cudaMalloc(&scratch, sizeof(int) * (5 * (size_t)n + 16)));
+    CK(scratch_ints(P, 5 * (size_t)n + 16, &scratch));
     unsigned long long* words = (unsigned long long*)scratch;
     int* qend = scratch + 6;
     int* nlev_dev = scratch + 10;
@@ -390,7 +424,6 @@ sptrsv_status_t kahn_levels(sptrsv_plan_t P, const int* ptr, const int* idx, con
             ++level;
         }
     }
-    cudaFree(scratch);
     if (e != cudaSuccess) return cuda_fail(e);
     int row = -1;
     ST(take_status(P, s, &row));
@@ -410,7 +443,7 @@ sptrsv_status_t build_levels(sptrsv_plan_t P, const int* ptr, const int* idx, bo
                              Levels& L, cudaStream_t s, int method = SPTRSV_ANALYSIS_AUTO,
                              const int* dptr = nullptr, const int* didx = nullptr) {
     const int n = P->n;
-    CK(cudaMalloc(&L.lev, sizeof(int) * (size_t)n));
+    if (!L.lev) CK(cudaMalloc(&L.lev, sizeof(int) * (size_t)n));
     CK(cudaMemsetAsync(L.lev, 0xff, sizeof(int) * (size_t)n, s));
     CK(cudaMemsetAsync(P->counters, 0, 2 * sizeof(int), s));
     int nlev = -1;
@@ -473,14 +506,13 @@ sptrsv_status_t level_sets(sptrsv_plan_t P, const int* ptr, Levels& L, int nlev,
     const int n = P->n;
     int row = -1;
     L.nlev = nlev;
-    CK(cudaMalloc(&L.ilev, sizeof(int) * (size_t)(nlev + 1)));
-    CK(cudaMalloc(&L.jlev, sizeof(int) * (size_t)n));
-    CK(cudaMalloc(&L.ipos, sizeof(int) * (size_t)n));
+    if (!L.ilev) CK(cudaMalloc(&L.ilev, sizeof(int) * (size_t)(nlev + 1)));
+    if (!L.jlev) CK(cudaMalloc(&L.jlev, sizeof(int) * (size_t)n));
+    if (!L.ipos) CK(cudaMalloc(&L.ipos, sizeof(int) * (size_t)n));
     int* count = nullptr;
     int* scratch = nullptr;
     const int hist_n = radix_hist_entries(n);
-    const size_t scratch_ints = (size_t)nlev + 4 * (size_t)n + 2 * (size_t)hist_n;
-    CK(cudaMalloc(&scratch, sizeof(int) * scratch_ints));
+    CK(scratch_ints(P, (size_t)nlev + 4 * (size_t)n + 2 * (size_t)hist_n, &scratch));
     count = scratch;
     int* k_a = count + nlev;
     int* v_a = k_a + n;
@@ -491,10 +523,10 @@ sptrsv_status_t level_sets(sptrsv_plan_t P, const int* ptr, Levels& L, int nlev,
     sptrsv_status_t rc = SPTRSV_OK;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int) * (size_t)nlev, s);
     if (e == cudaSuccess) e = launch_histogram(L.lev, n, count, nlev, P->status, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(count, L.ilev, nlev, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(count, L.ilev, nlev, P->scan_sums, s);
     if (e == cudaSuccess)
         e = radix_sort_values(L.lev, nullptr, n, bits_for(nlev - 1), L.jlev, k_a, v_a, k_b, v_b,
-                              hist, hist_scan, P->status, s);
+                              hist, hist_scan, P->scan_sums, P->status, s);
     if (e == cudaSuccess) e = launch_verify_levels(n, nlev, L.lev, L.ilev, L.jlev, P->status, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(P->counters + 2, 0, sizeof(int), s);
     if (e == cudaSuccess) e = launch_max_length(n, ptr, P->counters + 2, s);
@@ -507,7 +539,6 @@ sptrsv_status_t level_sets(sptrsv_plan_t P, const int* ptr, Levels& L, int nlev,
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) rc = cuda_fail(e);
-    cudaFree(scratch);
     if (rc == SPTRSV_OK) rc = take_status(P, s, &row);
     // jlev is now known to be a permutation: invert it for level-order tiles.
     if (rc == SPTRSV_OK) {
@@ -523,6 +554,7 @@ sptrsv_status_t build_transpose_pattern(sptrsv_plan_t P, cudaStream_t s);
 sptrsv_status_t build_transpose(sptrsv_plan_t P, cudaStream_t s) {
     if (P->has_trans) return SPTRSV_OK;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
+    ScratchScope scope(P);
     ST(build_transpose_pattern(P, s));
     ST(build_levels(P, P->tptr, P->tidx, !P->upper, P->trn, s, SPTRSV_ANALYSIS_AUTO, P->rowptr,
                     P->colidx));
@@ -535,17 +567,9 @@ sptrsv_status_t build_transpose_pattern(sptrsv_plan_t P, cudaStream_t s) {
     if (P->has_tpattern) return SPTRSV_OK;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     const int n = P->n, nnz = P->nnz;
-    cudaFree(P->tptr);  // left over from a failed attempt, if any
-    cudaFree(P->tidx);
-    cudaFree(P->tmap);
-    P->tptr = P->tidx = P->tmap = nullptr;
-    CK(cudaMalloc(&P->tptr, sizeof(int) * (size_t)(n + 1)));
-    CK(cudaMalloc(&P->tidx, sizeof(int) * (size_t)(nnz > 0 ? nnz : 1)));
-    CK(cudaMalloc(&P->tmap, sizeof(int) * (size_t)(nnz > 0 ? nnz : 1)));
     const int hist_n = radix_hist_entries(nnz);
-    const size_t scratch_ints = (size_t)n + 5 * (size_t)nnz + 2 * (size_t)hist_n;
     int* scratch = nullptr;
-    CK(cudaMalloc(&scratch, sizeof(int) * scratch_ints));
+    CK(scratch_ints(P, (size_t)n + 5 * (size_t)nnz + 2 * (size_t)hist_n, &scratch));
     int* count = scratch;
     int* k_a = count + n;
     int* v_a = k_a + nnz;
@@ -556,14 +580,13 @@ sptrsv_status_t build_transpose_pattern(sptrsv_plan_t P, cudaStream_t s) {
     int* hist_scan = hist + hist_n;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int) * (size_t)n, s);
     if (e == cudaSuccess) e = launch_histogram(P->colidx, nnz, count, n, P->status, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(count, P->tptr, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(count, P->tptr, n, P->scan_sums, s);
     if (e == cudaSuccess)
         e = radix_sort_values(P->colidx, nullptr, nnz, bits_for(n - 1), P->tmap, k_a, v_a, k_b,
-                              v_b, hist, hist_scan, P->status, s);
+                              v_b, hist, hist_scan, P->scan_sums, P->status, s);
     if (e == cudaSuccess) e = launch_row_of_entries(n, P->rowptr, rowof, s);
     if (e == cudaSuccess) e = launch_gather(rowof, nnz, P->tmap, nnz, P->tidx, P->status, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(scratch);
     if (e != cudaSuccess) return cuda_fail(e);
     int row = -1;
     sptrsv_status_t rc = take_status(P, s, &row);
@@ -637,7 +660,7 @@ sptrsv_status_t build_chain(sptrsv_plan_t P, bool trans, int lanes, cudaStream_t
     if (rc == SPTRSV_OK && (nslev < 1 || nslev > nseg)) rc = SPTRSV_ERR_INTERNAL;
     if (rc == SPTRSV_OK) {
         e = radix_sort_values(slev, nullptr, nseg, bits_for(nslev - 1), torder, k_a, v_a, k_b,
-                              v_b, hist, hist_scan, P->status, s);
+                              v_b, hist, hist_scan, P->scan_sums, P->status, s);
         if (e == cudaSuccess)
             e = launch_verify_segments(n, R, ptr, idx, upper, slev, nslev, P->status, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -683,7 +706,7 @@ sptrsv_status_t build_permuted(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaMalloc(&xp, esize * (size_t)n);
     if (e == cudaSuccess) e = cudaMalloc(&lens, sizeof(int) * (size_t)n);
     if (e == cudaSuccess) e = launch_ordered_lengths(n, ptr, L.jlev, lens, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(lens, pptr, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(lens, pptr, n, P->scan_sums, s);
     if (e == cudaSuccess)
         e = launch_permute_rows(P->f64, n, ptr, idx, vmap, P->vals, L.jlev, L.ipos, pptr, pidx,
                                 pvals, P->num_sms * 16, s, copy_diag(P, trans),
@@ -895,14 +918,14 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaMemsetAsync(depth, 0, sizeof(int) * N, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(counters, 0, sizeof(int) * 8, s);
     if (e == cudaSuccess) e = launch_part_spans(n, ptr, idx, upper, diff, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(diff, cover, n + 1, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(diff, cover, n + 1, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_block_flags(n, cover, bflag, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(bflag, bscan, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(bflag, bscan, n, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_flag_scatter(n, bflag, bscan, bstart, s);
     if (e == cudaSuccess) e = launch_block_depth(n, upper, L.lev, bscan, depth, s);
     // parts, numbered in order of substitution
     if (e == cudaSuccess) e = launch_part_flags(n, S, bscan, bstart, pflag, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(pflag, pscan, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(pflag, pscan, n, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_flag_scatter(n, pflag, pscan, pstart, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&nb, bscan + n, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&np, pscan + n, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -926,30 +949,29 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
                                       pkey, s);
         if (e == cudaSuccess)
             e = radix_sort_values(pkey, nullptr, np, bits_for(2 * maxdepth + 1), horder, k_a, v_a,
-                                  k_b, v_b, hist, hist_scan, P->status, s);
+                                  k_b, v_b, hist, hist_scan, P->scan_sums, P->status, s);
     } else if (e == cudaSuccess) {
         e = launch_part_depth_keys(np, maxdepth, pstart, bscan, depth, pkey, s);
     }
     if (e == cudaSuccess && order != 3)
         e = radix_sort_values(pkey, nullptr, np, bits_for(maxdepth),
-                              by_piece ? horder1 : horder, k_a, v_a, k_b, v_b, hist, hist_scan,
-                              P->status, s);
+                              by_piece ? horder1 : horder, k_a, v_a, k_b, v_b, hist, hist_scan, P->scan_sums, P->status, s);
     if (by_piece) {
         if (e == cudaSuccess) e = launch_part_piece(np, pstart, bscan, bstart, pscan, piece, s);
         if (e == cudaSuccess) e = launch_gather(piece, np, horder1, np, pkey2, P->status, s);
         if (e == cudaSuccess)
             e = radix_sort_values(pkey2, horder1, np, bits_for(np - 1), horder, k_a, v_a, k_b,
-                                  v_b, hist, hist_scan, P->status, s);
+                                  v_b, hist, hist_scan, P->scan_sums, P->status, s);
     }
     if (e == cudaSuccess) e = launch_inverse_perm(horder, np, prank, s);
     if (e == cudaSuccess) e = launch_part_sizes(n, np, upper, horder, pstart, psize, qrow, counters,
                                                s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(psize, qpart, np, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(psize, qpart, np, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_row_part_keys(n, L.jlev, upper, pscan, prank, rowkey, s);
     // rows by part (hand-out order), by level inside a part
     if (e == cudaSuccess)
         e = radix_sort_values(rowkey, L.jlev, n, bits_for(np - 1), qord, k_a, v_a, k_b, v_b,
-                              hist, hist_scan, P->status, s);
+                              hist, hist_scan, P->scan_sums, P->status, s);
     if (e == cudaSuccess) e = launch_inverse_perm(qord, n, qipos, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&maxpart, counters, sizeof(int),
                                               cudaMemcpyDeviceToHost, s);
@@ -1005,10 +1027,10 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     if (e == cudaSuccess) e = cudaMalloc(&q.grp_ptr, sizeof(int) * ((size_t)L.qnparts + 1));
     if (e == cudaSuccess) e = launch_run_flags(n, L.qord, L.lev, flag, s);
     if (e == cudaSuccess) e = launch_part_flag_starts(L.qnparts, L.qpart, flag, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(flag, scan, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(flag, scan, n, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_flag_scatter(n, flag, scan, rstart, s);
     if (e == cudaSuccess) e = launch_group_flags(n, 32 / lanes, scan, rstart, gflag, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(gflag, scan, n, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(gflag, scan, n, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_part_groups(L.qnparts, L.qpart, scan, q.grp_ptr, s);
     if (e == cudaSuccess) e = launch_flag_scatter(n, gflag, scan, flag, s);
     if (e == cudaSuccess)
@@ -1020,7 +1042,7 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     if (e == cudaSuccess) e = cudaMalloc(&q.grp, sizeof(int4) * (size_t)q.ngroups);
     const SliceParams sp = slice_params(P, trans, q);
     if (e == cudaSuccess) e = launch_group_shapes(sp, lanes, gstart, q.grp, rstart, s);
-    if (e == cudaSuccess) e = launch_exclusive_scan(cnt, base, q.ngroups, s);
+    if (e == cudaSuccess) e = launch_exclusive_scan(cnt, base, q.ngroups, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_group_bases(q.ngroups, base, q.grp, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&h[1], base + q.ngroups, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -1488,12 +1510,39 @@ sptrsv_status_t sptrsv_analyze(int n, int nnz, const int* d_rowptr, const int* d
     P->spin.hot = (int)env_ll("SPTRSV_SPIN_HOT", 256);
     P->spin.max_ns = (unsigned)env_ll("SPTRSV_SPIN_MAX_NS", 128);
     sptrsv_status_t rc = SPTRSV_OK;
-    e = cudaMalloc(&P->counters, 4 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&P->status, sizeof(unsigned long long));
+    {   // parts of whole 128-byte lines
+        size_t at = 0;
+        auto part = [&](size_t ints) {
+            const size_t here = at;
+            at += (ints + 31) / 32 * 32;
+            return here;
+        };
+        const size_t N = (size_t)n, Z = (size_t)nnz;
+        const size_t o_status = part(2), o_counters = part(4), o_sums = part(kScanSums);
+        const size_t o_tptr = part(N + 1), o_tidx = part(Z), o_tmap = part(Z);
+        // at most n levels: nlev + 1 <= n + 1 entries
+        const size_t o_lev = part(N), o_ilev = part(N + 1), o_jlev = part(N), o_ipos = part(N);
+        e = cudaMalloc(&P->arena, sizeof(int) * at);
+        if (e == cudaSuccess) {
+            int* const base = (int*)P->arena;
+            P->status = (unsigned long long*)(base + o_status);
+            P->counters = base + o_counters;
+            P->scan_sums = base + o_sums;
+            P->tptr = base + o_tptr;
+            P->tidx = base + o_tidx;
+            P->tmap = base + o_tmap;
+            P->fwd.lev = base + o_lev;
+            P->fwd.ilev = base + o_ilev;
+            P->fwd.jlev = base + o_jlev;
+            P->fwd.ipos = base + o_ipos;
+            P->fwd.in_arena = true;
+        }
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(P->counters, 0, 4 * sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(P->status, 0xff, sizeof(unsigned long long), s);
     if (e != cudaSuccess) rc = cuda_fail(e);
     if (rc == SPTRSV_OK && n > 0) {
+        ScratchScope scope(P);
         e = launch_validate(n, nnz, d_rowptr, d_colidx, d_vals, P->f64, P->upper, P->unit,
                             P->status, P->num_sms * 32, s);
         if (e != cudaSuccess) rc = cuda_fail(e);
@@ -1531,6 +1580,7 @@ sptrsv_status_t sptrsv_reanalyze(sptrsv_plan_t plan, int transpose, sptrsv_analy
     cudaStream_t s = (cudaStream_t)stream;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     if (transpose) ST(build_transpose(P, s));
+    ScratchScope scope(P);
     CK(cudaStreamSynchronize(s));
     const auto t0 = std::chrono::steady_clock::now();
     const bool kahn = method != SPTRSV_ANALYSIS_SWEEP;

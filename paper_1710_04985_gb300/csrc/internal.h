@@ -264,15 +264,18 @@ cudaError_t launch_verify_segments(int n, int R, const int* ptr, const int* idx,
 // an internal error in *status and skipped.
 cudaError_t launch_histogram(const int* keys, int m, int* count, int bins,
                              unsigned long long* status, cudaStream_t s);
-// out[0..m]: exclusive prefix sums of in[0..m-1], out[m] = total.
-cudaError_t launch_exclusive_scan(const int* in, int* out, int m, cudaStream_t s);
+// out[0..m]: exclusive prefix sums of in[0..m-1], out[m] = total.  sums: scratch
+// of kScanSums ints, one scan at a time.
+constexpr int kScanSums = 1025;
+cudaError_t launch_exclusive_scan(const int* in, int* out, int m, int* sums, cudaStream_t s);
 // Stable LSD radix sort of (keys, values = vals_in or the identity) by the
 // low `bits` bits of the keys; sorted values land in vals_out.  Scratch:
-// 4 int arrays of m entries and one of radix_hist_entries(m) entries (x2).
+// 4 int arrays of m entries, one of radix_hist_entries(m) entries (x2) and the
+// scan's sums.
 int radix_hist_entries(int m);
 cudaError_t radix_sort_values(const int* keys_in, const int* vals_in, int m, int bits,
                               int* vals_out, int* k_a, int* v_a, int* k_b, int* v_b,
-                              int* hist, int* hist_scan, unsigned long long* status,
+                              int* hist, int* hist_scan, int* sums, unsigned long long* status,
                               cudaStream_t s);
 cudaError_t launch_iota(int* out, int m, cudaStream_t s);
 cudaError_t launch_row_of_entries(int n, const int* ptr, int* rowof, cudaStream_t s);
