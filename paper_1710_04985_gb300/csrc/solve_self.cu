@@ -30,8 +30,11 @@
 // Measured against the kernel before (every row folded and published by itself,
 // tickets of any levels in one round loop), plan defaults, FP64, us: 7-point
 // 61 x 47 x 53 in place 205 -> 182 and its adjoint 210 -> 182, 27-point of that
-// size 467 -> 381, 128^3 ILU(0) L 570 -> 548; general matrix of 150001 rows 5656 ->
-// 5300 and its adjoint 5688 -> 5231 (16 lanes; 32 lanes 4858 -> 4810).
+// size 467 -> 354, 128^3 ILU(0) L 570 -> 536; general matrix of 150001 rows 5656 ->
+// 5300 and its adjoint 5688 -> 4927 (16 lanes; 32 lanes 4858 -> 4670), of 600001 rows
+// with 32 lanes 18924 -> 18425.  Of these, two entries a lane instead of four at
+// 16 and 32 lanes and a lane sum with at most three branches give the last 3 to 8 %
+// on the 27-point and the general ones.
 #include "internal.h"
 
 namespace sptrsv {
@@ -76,6 +79,13 @@ namespace {
 
 constexpr int kMaxSelfBlock = 512;  // larger blocks run as several of this size
 constexpr int kSelfHot = 64;        // polls of one wait before the warp backs off
+// Entries a lane holds at once: groups of 16 and 32 lanes hold an average row in one
+// or two, and every further slot costs its instructions in each polling round
+// (general 150001 rows, 32 lanes 4811 us with four, 4670 with two).
+template <int W>
+struct ChunkOf {
+    static constexpr int E = W >= 16 ? 2 : kChunk;
+};
 
 __device__ __forceinline__ double lds_relaxed(const double* p) { return *(const volatile double*)p; }
 __device__ __forceinline__ float lds_relaxed(const float* p) { return *(const volatile float*)p; }
@@ -170,6 +180,31 @@ __device__ __forceinline__ void scale_entries(const SolveParams& p, T dinv, cons
         }
 }
 
+// group_sum_span (the same sums in the same order) with at most three branches
+// instead of one per level of the butterfly.
+template <int OFF, typename T>
+__device__ __forceinline__ T sum_from(T v) {
+    v += __shfl_xor_sync(0xffffffffu, v, OFF);
+    if constexpr (OFF > 1) v = sum_from<OFF / 2>(v);
+    return v;
+}
+template <int W, typename T>
+__device__ __forceinline__ T row_sum(T v, int span) {
+    if constexpr (W == 1) return v;
+    if constexpr (W == 2) return span > 1 ? sum_from<1>(v) : v;
+    if constexpr (W >= 4) {
+        if (span > 4) {
+            if constexpr (W >= 32)
+                if (span > 16) return sum_from<16>(v);
+            if constexpr (W >= 16)
+                if (span > 8) return sum_from<8>(v);
+            if constexpr (W >= 8) return sum_from<4>(v);
+        }
+        if (span > 2) return sum_from<2>(v);
+        return span > 1 ? sum_from<1>(v) : v;
+    }
+}
+
 // Whether the warp takes the rows of a ticket as one, where the matrix as a
 // whole does not say so (SolveParams::rows_alike): equally many chunks of
 // entries, lengths within a factor of about two (unless there are only two
@@ -185,8 +220,8 @@ __device__ __forceinline__ bool alike(bool has, int len, int lev) {
     const int top = __reduce_max_sync(FULL, has ? lev : -1);
     const int low = __reduce_min_sync(FULL, has ? lev : 0x7fffffff);
     if (top - low >= kLevels) return false;
-    if ((most + W * kChunk - 1) / (W * kChunk) != (least + W * kChunk - 1) / (W * kChunk))
-        return false;
+    constexpr int C = W * ChunkOf<W>::E;
+    if ((most + C - 1) / C != (least + C - 1) / C) return false;
     return W >= 16 || most <= 2 * least + 2;
 }
 
@@ -345,7 +380,7 @@ __global__ void __launch_bounds__(kMaxSelfBlock, 1)
     extern __shared__ __align__(16) unsigned char self_smem[];
     __shared__ int s_next;
     constexpr int R = 32 / W;
-    constexpr int E = kChunk;
+    constexpr int E = ChunkOf<W>::E;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int grp = lane / W;
@@ -391,6 +426,7 @@ __global__ void __launch_bounds__(kMaxSelfBlock, 1)
         const int span = warp_span<W>(r.has, r.end - r.beg);
         const long long own = PERM ? r.k : (long long)r.i * ldp;
         bool todo = r.has, ok = true;
+        const bool out = r.has && sl == 0 && r.i != p.withhold;
         while (true) {
             // the rows of the lowest level that is left
             bool act = todo;
@@ -447,8 +483,8 @@ __global__ void __launch_bounds__(kMaxSelfBlock, 1)
                     }
             }
             if (!ok) break;
-            const T tot = group_sum_span<W>(r.sum, FULL, span);
-            if (act && sl == 0 && r.i != p.withhold) {
+            const T tot = row_sum<W>(r.sum, span);
+            if (act && out) {
                 const T val = publishable(tot);
                 if (SMALL)
                     *(volatile T*)(xpub + own) = val;
