@@ -1056,6 +1056,18 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
         e = cudaMalloc(&q.cols, sizeof(int) * slots);
         if (e == cudaSuccess) e = cudaMalloc(&q.vals, esize * slots);
         if (e == cudaSuccess && !P->unit) e = cudaMalloc(&q.dinv, esize * N);
+        if (e == cudaErrorMemoryAllocation) {
+            // no room for the padding: the level-ordered copy takes less
+            cudaGetLastError();
+            cudaFree(q.cols);
+            cudaFree(q.vals);
+            q.cols = nullptr;
+            q.vals = nullptr;
+            q.wide = true;
+            e = cudaSuccess;
+        }
+    }
+    if (e == cudaSuccess && !q.wide) {
         if (e == cudaSuccess)
             e = launch_fill_slices(P->f64, sp, lanes, q.grp, P->vals, q.cols, q.vals, q.dinv, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1193,8 +1205,23 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     // for the FP32 solves of a refined F64 plan (f64 != P->f64).
     if (f64 != P->f64 && !f32_of_f64) return SPTRSV_ERR_INVALID_ARG;
     bool parts = algo == SPTRSV_ALGO_SELF_PARTITIONED && !mrhs;
+    void* stand_in = nullptr;
     if (parts) {
         ST(build_parts(P, trans, s));
+        // While s is being captured a copy cannot be built for another width than
+        // the one prepared: that solve runs in place (bitwise the same result),
+        // with the publication buffer of the parts to keep b in.
+        const Levels& Lq = trans ? P->trn : P->fwd;
+        const Levels::Slices& q = Lq.qs[log2_lanes(lanes)];
+        if (!f32_of_f64 && (!q.built || (q.wide && !Lq.pptr)) && capturing(s))
+            for (const Levels::Slices& o : Lq.qs)
+                if (o.built) stand_in = Lq.xq;
+        if (stand_in) {
+            algo = SPTRSV_ALGO_SELF;
+            parts = false;
+        }
+    }
+    if (parts) {
         ST(build_slices(P, trans, lanes, s));
         parts = !(trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].wide;
         if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
@@ -1394,8 +1421,9 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         const size_t esize = f64 ? sizeof(double) : sizeof(float);
         void* bcopy = nullptr;
         if (x == b) {  // in place: keep b aside, x becomes the publication buffer
-            ST(ensure_bytes(&P->bcopy, &P->bcopy_bytes, esize * (size_t)P->n * nrhs, s));
-            bcopy = P->bcopy;
+            if (!stand_in)
+                ST(ensure_bytes(&P->bcopy, &P->bcopy_bytes, esize * (size_t)P->n * nrhs, s));
+            bcopy = stand_in ? stand_in : P->bcopy;
             p.b = bcopy;
             p.ldb = nrhs;
         }

@@ -116,3 +116,23 @@ def test_a_value_that_never_comes_holds_up_only_its_dependents(lanes, cluster):
         p.withhold_row(-1)
         assert relerr(p.solve(torch.tensor(b, device=dev()), algo="partitioned"), ref) <= TOL64
         assert p.status() == (0, -1)
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+def test_capture_at_a_width_that_was_not_prepared(in_place):
+    """A captured solve cannot build the copy of another width: it runs on what is
+    there, also in place, with the result of that width."""
+    A = synth.laplacian_triangles((13, 17, 9), 7)[0]
+    b = torch.tensor(synth.uniform(A.n, 73), device=dev())
+    with plan_for(A) as p:
+        p.set_tuning(1, 128, 0)
+        p.prepare("partitioned")
+        p.set_tuning(4, 128, 0)
+        x = b.clone() if in_place else torch.empty_like(b)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            p.solve(x if in_place else b, out=x, algo="partitioned")
+        g.replay()
+        assert torch.equal(x, p.solve(b, algo="self"))
+        assert torch.equal(x, p.solve(b, algo="partitioned"))
+        assert p.status() == (0, -1)
