@@ -249,6 +249,9 @@ struct sptrsv_plan_s {
     // multi-RHS launch shape: width (0: chosen from nrhs), block (0: the
     // single-RHS one), grid cap (-1: the single-RHS one)
     int mrhs_lanes = 0, mrhs_block = 0, mrhs_max_blocks = -1;
+    // largest cluster of each solve_cluster.cu kernel (-1: not asked yet):
+    // element type, log2 lanes, in place / through the map / level-ordered copy
+    signed char cluster_cap[2][6][3];
     int tile_rows = 2048;
     bool tile_level_order = false;
     int part_rows = 0;   // partitioned solve: rows per part (0: automatic)
@@ -846,6 +849,22 @@ bool small_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes) {
     return (long long)P->n * lanes <= 32ll * kSmallGroups * (f64 ? 1 : 2) * L.nlev;
 }
 
+// Blocks of the cluster that a single-RHS solve of the in-place or level-ordered
+// form runs on, 0: the whole GPU.  On a cluster a hop is shorter, but every row is
+// stored into each of its blocks and 16 SMs fold: an average level must hold at most
+// kClusterGroups row groups (32 / lanes rows) of 16 or 32 lanes.  (us, whole GPU and
+// cluster: general 150001 rows, 28 groups a level, 4670 and 3236; 14 groups 5300 and
+// 4350; 27-point 61 x 47 x 53, 16 lanes, 210 groups, 354 and 835.  Narrower groups mean
+// more stores a level: 5-point 1024 x 1024 with 2 lanes, 32 groups, 2046 and 2145.)
+constexpr int kClusterGroups = 32;
+int cluster_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes, int max_blocks, bool map,
+                  bool perm) {
+    if (lanes < 16 || (long long)P->n * lanes > 32ll * kClusterGroups * L.nlev) return 0;
+    signed char& cap = P->cluster_cap[f64 ? 1 : 0][log2_lanes(lanes)][perm ? 2 : map ? 1 : 0];
+    if (cap < 0) cap = (signed char)cluster_blocks(f64, lanes, map, perm);
+    return max_blocks > 0 && max_blocks < cap ? 0 : cap;
+}
+
 // The part size of the next partitioned solve: the plan's setting or the
 // rows divided evenly over the SMs, at most max_part_rows.
 int resolve_part_rows(sptrsv_plan_t P) {
@@ -1382,7 +1401,9 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         p.xp = f32_of_f64 ? L.xp32 : L.xp;
         p.prescaled = P->unit ? 0 : 1;
         const bool small = !blocked && small_solve(P, L, f64, lanes);
-        if (!small)
+        const int on_cluster =
+            blocked || small ? 0 : cluster_solve(P, L, f64, lanes, max_blocks, false, true);
+        if (!small && !on_cluster)
             CK(launch_prep_self(f64, P->n, 1, p.xp, 1, nullptr, 0, nullptr, P->counters,
                                 P->num_sms * 8, s));
         const int R = 32 / lanes;
@@ -1391,6 +1412,10 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         if (small) {
             ST(prof_begin(P, s));
             CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
+            ST(prof_end(P, s));
+        } else if (on_cluster) {
+            ST(prof_begin(P, s));
+            CK(launch_cluster_k1(f64, lanes, p, on_cluster, s));
             ST(prof_end(P, s));
         } else if (blocked) {
             const long long tiles = ((long long)P->n + P->tile_rows - 1) / P->tile_rows;
@@ -1411,10 +1436,18 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             CK(launch_self_k1(f64, lanes, p, (int)grid, block, s));
             ST(prof_end(P, s));
         }
-        launches = small ? 1 : 2;
+        launches = small || on_cluster ? 1 : 2;
     } else if (algo == SPTRSV_ALGO_SELF && !mrhs && small_solve(P, L, f64, lanes)) {
         ST(prof_begin(P, s));
         CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
+        ST(prof_end(P, s));
+        launches = 1;
+    } else if (const int on_cluster =
+                   algo == SPTRSV_ALGO_SELF && !mrhs
+                       ? cluster_solve(P, L, f64, lanes, max_blocks, p.vmap != nullptr, false) : 0) {
+        p.ipos = L.ipos;
+        ST(prof_begin(P, s));
+        CK(launch_cluster_k1(f64, lanes, p, on_cluster, s));
         ST(prof_end(P, s));
         launches = 1;
     } else {
@@ -1514,6 +1547,7 @@ sptrsv_status_t sptrsv_analyze(int n, int nnz, const int* d_rowptr, const int* d
     cudaStream_t s = (cudaStream_t)stream;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     sptrsv_plan_t P = new sptrsv_plan_s();
+    memset(P->cluster_cap, -1, sizeof(P->cluster_cap));
     cudaError_t e = cudaGetDevice(&P->device);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, P->device);

@@ -30,8 +30,8 @@ struct SolveParams {
     unsigned long long* status;
     SpinPolicy spin;
     int withhold;         // test hook: row whose result is never published (-1: none)
-    const int* ipos;      // tiled solve in level order: position of each row in jlev
-                          // (nullptr: tiles follow the substitution order)
+    const int* ipos;      // tiled solve in level order, solve on one cluster: position of
+                          // each row in jlev (tiles: nullptr: in substitution order)
     int kbeg, cnt;        // level-scheduled: this launch's slice of jlev
     void* xp;             // level-ordered solve: publication buffer in position
                           // order (nullptr: rows publish to x itself)
@@ -147,6 +147,12 @@ int self_k1_blocks_per_sm(bool f64, int lanes, bool map, bool perm, int block);
 // prep launch: b is read before x is written, in place too.
 cudaError_t launch_self_small(bool f64, int lanes, const SolveParams& p, int block,
                               cudaStream_t s);
+// The whole system on one cluster of nblocks blocks (solve_cluster.cu; in place it
+// needs p.ipos, the position of each row); 16 or 32 lanes.  No prep launch either.
+cudaError_t launch_cluster_k1(bool f64, int lanes, const SolveParams& p, int nblocks,
+                              cudaStream_t s);
+// Blocks of the largest cluster that can run (0: none).
+int cluster_blocks(bool f64, int lanes, bool map, bool perm);
 
 // ---- partitioned solve (solve_parts.cu).  Positions t are in order of
 // substitution (row t of a lower system, row n-1-t of an upper one).
