@@ -60,7 +60,8 @@ KERNELS = {
     "chains": ("chain_solve_k1", "solve_chain.cu", None),
     "permuted": ("self_solve_k1", "solve_self.cu", "self_solve_k1_permuted_ilu0_7pt_128.md"),
     "blocked": ("blocked_solve_k1", "solve_blocked.cu", None),
-    "partitioned": ("part_solve_k1", "solve_partitioned.cuh", None),
+    "partitioned": ("part_solve_k1", "solve_partitioned.cuh",
+                    "part_solve_k1_ilu0_7pt_128.md"),
 }
 
 
