@@ -392,7 +392,9 @@ SPTRSV_API sptrsv_status_t sptrsv_refresh_values(sptrsv_plan_t plan, void *strea
  * max_blocks caps the persistent grid of the self-scheduled solve (0 = as
  * many as fit on the device at once; the default is 2 blocks per SM, which
  * keeps enough rows waiting ahead of the dependency frontier without
- * flooding L2 with polls).  Applies to the forward and the transposed
+ * flooding L2 with polls).  In-place and level-ordered solves of systems with
+ * narrow levels run in one block or on one cluster of 16 (a max_blocks of 1 to
+ * 15 keeps them off the cluster).  Applies to the forward and the transposed
  * solves.  Sets the shape of every algorithm (clearing the shapes set for
  * single algorithms by sptrsv_set_algo_tuning).  Multi-RHS solves have their
  * own launch shape (sptrsv_set_mrhs_tuning), by default this block size and
