@@ -430,14 +430,27 @@ cudaError_t launch_self_k1(bool f64, int lanes, const SolveParams& p, int grid, 
     });
 }
 
+// The shared memory that a one-block instance may ask for: the device's opt-in limit
+// less the room of its static variables, the same on every call.  The limit belongs to
+// the kernel on the device, not to a plan: a call that set its own smaller size could
+// come between the two steps of another thread's larger one, whose launch then fails.
+static cudaError_t small_limit(const void* k) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e == cudaSuccess
+               ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 128)
+               : e;
+}
+
 cudaError_t launch_self_small(bool f64, int lanes, const SolveParams& p, int block,
                               cudaStream_t s) {
     const size_t smem = (f64 ? 8 : 4) * (size_t)p.n;  // checked by the caller
     if (block > kMaxSelfBlock) block = kMaxSelfBlock;
     return self_any(f64, lanes, !p.xp && p.vmap, p.xp != nullptr, true, [&](auto k) {
         if (smem > 48 * 1024 - 256) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
+            const cudaError_t e = small_limit((const void*)k);
             if (e != cudaSuccess) return e;
         }
         k<<<1, block, smem, s>>>(p);

@@ -1,0 +1,133 @@
+"""What the library asks of the CUDA runtime, seen and steered by a shim in front
+of libcudart: limits of a kernel that all plans of a process share.  The shim is
+preloaded into a child process, once for all tests."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SHIM = r"""
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <cuda_runtime_api.h>
+
+static void* find(const char* name) {
+    void* f = dlsym(RTLD_NEXT, name);   /* where libcudart is in the global scope */
+    return f ? f : dlsym(dlopen("libcudart.so.13", RTLD_LAZY | RTLD_NOLOAD), name);
+}
+#define REAL(f) __typeof__(&f) real = (__typeof__(&f))find(#f)
+
+/* limits: how often a kernel's shared memory was set below an earlier value */
+static const void* funcs[1024];
+static int values[1024], nfuncs, lowered;
+int shim_lowered(void) { return lowered; }
+
+cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) {
+    REAL(cudaFuncSetAttribute);
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+        int k = 0;
+        while (k < nfuncs && funcs[k] != f) ++k;
+        if (k == nfuncs && nfuncs < 1024) {
+            funcs[nfuncs++] = f;
+            values[k] = v;
+        }
+        if (k < nfuncs) {
+            if (v < values[k]) ++lowered;
+            values[k] = v;
+        }
+    }
+    return real(f, a, v);
+}
+"""
+
+CHILD = r"""
+import ctypes, json, sys
+sys.path[:0] = [sys.argv[1], sys.argv[1] + "/tests"]
+import torch
+import synth
+from gpu_util import dev, plan_for
+
+shim = ctypes.CDLL(sys.argv[2])
+out = {}
+
+
+def rhs(A):
+    return torch.tensor(synth.uniform(A.n, 7), device=dev())
+
+
+def one_block():
+    big, small = synth.lap2d_5pt_lower(60, 450), synth.lap2d_5pt_lower(60, 150)
+    with plan_for(big) as p, plan_for(small) as q:
+        for plan, A in ((p, big), (q, small), (p, big)):
+            plan.set_tuning(2, 256, 0)
+            plan.solve(rhs(A))
+            assert plan.last_launch_count == 1      # the one-block kernel
+    out["lowered"] = shim.shim_lowered()
+
+
+for f in (one_block,):
+    f()
+print(json.dumps(out))
+"""
+
+
+@pytest.fixture(scope="module")
+def seen(cuda_device, tmp_path_factory):
+    from paper_1710_04985_gb300 import build
+    d = tmp_path_factory.mktemp("shim")
+    (d / "shim.c").write_text(SHIM)
+    (d / "child.py").write_text(CHILD)
+    inc = os.path.join(os.path.dirname(build._cuda_lib_dir(build._nvcc())), "include")
+    so = str(d / "shim.so")
+    r = subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-I", inc, str(d / "shim.c"), "-o", so,
+                        "-ldl"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([sys.executable, str(d / "child.py"), ROOT, so], capture_output=True,
+                       text=True, timeout=300, env=dict(os.environ, LD_PRELOAD=so))
+    assert r.returncode == 0, r.stdout + r.stderr
+    return json.loads(r.stdout.splitlines()[-1])
+
+
+def test_one_block_solves_never_lower_the_limit_of_another_plan(seen):
+    """The limit belongs to the kernel, not to the plan: a smaller system must not
+    take away what a larger one, launched by another thread, is about to use."""
+    assert seen["lowered"] == 0
+
+
+def test_two_threads_with_plans_of_their_own(cuda_device):
+    """The calls of both are valid whatever the other one launches in between."""
+    import threading
+
+    import torch
+
+    import synth
+    from gpu_util import dev, plan_for
+    errors = []
+
+    def work(ny):
+        try:
+            A = synth.lap2d_5pt_lower(60, ny)
+            b = torch.tensor(synth.uniform(A.n, 7), device=dev())
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream), plan_for(A) as p:
+                p.set_tuning(2, 256, 0)
+                want = p.solve(b, algo="blocked")
+                x = torch.empty_like(b)
+                for _ in range(300):
+                    p.solve(b, out=x)
+                stream.synchronize()
+                assert torch.equal(x, want)
+        except Exception as e:
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(ny,)) for ny in (450, 150)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert errors == []
