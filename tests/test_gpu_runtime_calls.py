@@ -1,6 +1,6 @@
 """What the library asks of the CUDA runtime, seen and steered by a shim in front
-of libcudart: limits of a kernel that all plans of a process share.  The shim is
-preloaded into a child process, once for all tests."""
+of libcudart: limits of a kernel that all plans of a process share, and queries
+that fail.  The shim is preloaded into a child process, once for all tests."""
 import json
 import os
 import subprocess
@@ -43,6 +43,26 @@ cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v)
     }
     return real(f, a, v);
 }
+
+/* clusters: a size whose query fails, and the last one launched */
+static unsigned refused, launched;
+void shim_refuse_cluster(unsigned blocks) { refused = blocks; }
+unsigned shim_launched_cluster(void) { return launched; }
+static unsigned cluster_of(const cudaLaunchConfig_t* c) {
+    for (unsigned k = 0; k < c->numAttrs; ++k)
+        if (c->attrs[k].id == cudaLaunchAttributeClusterDimension)
+            return c->attrs[k].val.clusterDim.x;
+    return 1;
+}
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) {
+    REAL(cudaOccupancyMaxActiveClusters);
+    return refused && cluster_of(c) == refused ? cudaErrorInvalidClusterSize : real(n, f, c);
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
+    REAL(cudaLaunchKernelExC);
+    launched = cluster_of(c);
+    return real(c, f, args);
+}
 """
 
 CHILD = r"""
@@ -70,7 +90,24 @@ def one_block():
     out["lowered"] = shim.shim_lowered()
 
 
-for f in (one_block,):
+def cluster():
+    A = synth.general_lower(4000, 5)
+    b = rhs(A)
+    with plan_for(A) as p:
+        p.set_tuning(32, 256, 0)
+        want = p.solve(b, algo="blocked")
+        p.solve(b)
+        out["cluster_first"] = [p.last_launch_count, shim.shim_launched_cluster()]
+    shim.shim_refuse_cluster(16)
+    with plan_for(A) as p:
+        p.set_tuning(32, 256, 0)
+        got = p.solve(b)
+        out["cluster_refused"] = [p.last_launch_count, shim.shim_launched_cluster(),
+                                  bool(torch.equal(got, want))]
+    shim.shim_refuse_cluster(0)
+
+
+for f in (one_block, cluster):
     f()
 print(json.dumps(out))
 """
@@ -97,6 +134,11 @@ def test_one_block_solves_never_lower_the_limit_of_another_plan(seen):
     """The limit belongs to the kernel, not to the plan: a smaller system must not
     take away what a larger one, launched by another thread, is about to use."""
     assert seen["lowered"] == 0
+
+
+def test_a_cluster_size_that_cannot_be_asked_for_leaves_the_smaller_one(seen):
+    assert seen["cluster_first"] == [1, 16]
+    assert seen["cluster_refused"] == [1, 8, True]
 
 
 def test_two_threads_with_plans_of_their_own(cuda_device):
