@@ -317,23 +317,27 @@ cudaLaunchConfig_t cluster_config(int nblocks, size_t smem, cudaStream_t s,
 
 int cluster_blocks(bool f64, int lanes, bool map, bool perm) {
     int blocks = 0;
+    // only an error of these calls is cleared, not one that the caller's code left
+    auto asked = [](cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
+    };
     const cudaError_t rc = cluster_any(f64, lanes, map, perm, [&](auto k) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             2 * kWindowBytes);
+        cudaError_t e = asked(cudaFuncSetAttribute(
+            k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWindowBytes));
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = asked(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         if (e != cudaSuccess) return e;
         // a size that cannot be asked for is one that cannot run: the next smaller one may
         for (int c = kMaxCluster; c >= 8 && !blocks; c /= 2) {
             cudaLaunchAttribute attr[1];
             const cudaLaunchConfig_t cfg = cluster_config(c, 2 * kWindowBytes, nullptr, attr);
             int nb = 0;
-            e = cudaOccupancyMaxActiveClusters(&nb, k, &cfg);
+            e = asked(cudaOccupancyMaxActiveClusters(&nb, k, &cfg));
             if (e == cudaSuccess && nb > 0) blocks = c;
         }
         return blocks ? cudaSuccess : e;
     });
-    cudaGetLastError();
     return rc == cudaSuccess ? blocks : 0;
 }
 

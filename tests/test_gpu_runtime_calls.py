@@ -24,8 +24,9 @@ static void* find(const char* name) {
 
 /* limits: how often a kernel's shared memory was set below an earlier value */
 static const void* funcs[1024];
-static int values[1024], nfuncs, lowered;
+static int values[1024], nfuncs, lowered, last_errors;
 int shim_lowered(void) { return lowered; }
+int shim_last_errors(void) { return last_errors; }
 
 cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) {
     REAL(cudaFuncSetAttribute);
@@ -42,6 +43,12 @@ cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v)
         }
     }
     return real(f, a, v);
+}
+
+cudaError_t cudaGetLastError(void) {
+    REAL(cudaGetLastError);
+    ++last_errors;
+    return real();
 }
 
 /* clusters: a size whose query fails, and the last one launched */
@@ -98,6 +105,16 @@ def cluster():
         want = p.solve(b, algo="blocked")
         p.solve(b)
         out["cluster_first"] = [p.last_launch_count, shim.shim_launched_cluster()]
+        counts = []
+        for _ in range(2):
+            before = shim.shim_last_errors()
+            p.solve(b)
+            counts.append(shim.shim_last_errors() - before)
+    with plan_for(A) as p:                          # a plan that has not asked yet
+        p.set_tuning(32, 256, 0)
+        before = shim.shim_last_errors()
+        p.solve(b)
+        out["last_errors"] = [shim.shim_last_errors() - before, counts[1]]
     shim.shim_refuse_cluster(16)
     with plan_for(A) as p:
         p.set_tuning(32, 256, 0)
@@ -139,6 +156,11 @@ def test_one_block_solves_never_lower_the_limit_of_another_plan(seen):
 def test_a_cluster_size_that_cannot_be_asked_for_leaves_the_smaller_one(seen):
     assert seen["cluster_first"] == [1, 16]
     assert seen["cluster_refused"] == [1, 8, True]
+
+
+def test_asking_for_the_cluster_size_clears_no_error_of_the_caller(seen):
+    first, later = seen["last_errors"]
+    assert first == later
 
 
 def test_two_threads_with_plans_of_their_own(cuda_device):
