@@ -1,0 +1,32 @@
+// Index arithmetic of the solve kernels at the limit of their int indices (n and nnz
+// up to SPTRSV_MAX_SIZE, 256 below 2^31).  Plain C++, so that it can be checked on the
+// host with the limit's own numbers.
+#pragma once
+
+#ifdef __CUDACC__
+#define SPTRSV_HD __host__ __device__ __forceinline__
+#else
+#define SPTRSV_HD inline
+#endif
+
+namespace sptrsv {
+
+// A lane's cursor over the entries [.., end) of its row, `step` further on.  The lanes
+// of a warp go through chunks together, for as long as its longest row lasts: the
+// cursor of a lane whose row has ended stays where it is, less than a step past the
+// end, instead of running on by the length of its neighbour's row.
+SPTRSV_HD int advance(int cursor, int step, int end) {
+    return cursor < end ? cursor + step : cursor;
+}
+
+// An entry index that a kernel forms is at most this far past the end of its row (the
+// kernels assert it for their chunks): it stays an int at the limit.
+constexpr int kCursorAhead = 255;
+
+// The furthest for chunks of `slots` slots of `lanes` entries: a cursor that has just
+// been advanced past the end, the chunk after its own, the last slot of it.
+constexpr int cursor_ahead(int lanes, int slots) {
+    return (lanes * slots - 1) + lanes * slots + lanes * (slots - 1);
+}
+
+}  // namespace sptrsv

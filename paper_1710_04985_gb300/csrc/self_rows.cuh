@@ -1,6 +1,7 @@
 // What the single-RHS kernels of the in-place and level-ordered forms do with a row
 // of a ticket (solve_self.cu, solve_cluster.cu): 32 / W rows per warp, W lanes each.
 #pragma once
+#include "cursor.h"
 #include "internal.h"
 
 namespace sptrsv {
@@ -12,6 +13,7 @@ namespace {
 template <int W>
 struct ChunkOf {
     static constexpr int E = W >= 16 ? 2 : kChunk;
+    static_assert(cursor_ahead(W, E) <= kCursorAhead, "entry index");
 };
 
 __device__ __forceinline__ double lds_relaxed(const double* p) { return *(const volatile double*)p; }

@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
                 start_row<T, W, MAP>(p, r, sl);
                 int c[E];
                 T a[E];
-                for (int q0 = r.beg + sl; __any_sync(FULL, act && q0 < r.end); q0 += W * E) {
+                for (int q0 = r.beg + sl; __any_sync(FULL, act && q0 < r.end);
+                     q0 = advance(q0, W * E, r.end)) {
                     load_entries<T, W, MAP, PERM, E>(p, r, q0, c, a);
                     scale_entries(p, r.dinv, c, a);
 #pragma unroll

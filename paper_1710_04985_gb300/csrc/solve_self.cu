@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kMaxSelfBlock, 1)
                     if (act) r.sum = fma(-a[e], v[e], r.sum);  // no entry: adds -0 * 0
                 }
                 if (!more) break;
-                q0 += W * E;
+                q0 = advance(q0, W * E, r.end);
 #pragma unroll
                 for (int e = 0; e < E; ++e)
                     if (act) {
