@@ -29,4 +29,10 @@ constexpr int cursor_ahead(int lanes, int slots) {
     return (lanes * slots - 1) + lanes * slots + lanes * (slots - 1);
 }
 
+// The start of the window of `rows` rows after the one at `base`, or n after the last
+// (base + rows may be past the largest int).
+SPTRSV_HD int next_window(int base, int rows, int n) {
+    return n - base > rows ? base + rows : n;
+}
+
 }  // namespace sptrsv

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
 
     bool slow = false;
     int buf = 0;
-    for (int base = 0; base < p.n; base += H, buf ^= 1) {
+    for (int base = 0; base < p.n; base = next_window(base, H, p.n), buf ^= 1) {
         const T* const ring = (const T*)ring_smem + buf * H;
         volatile int* const bail = &s_bail[buf];
         const unsigned to_win = to_ring + (unsigned)buf * (unsigned)kWindowBytes;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
                 }
             }
         };
-        if (base + H < p.n) {
+        if (next_window(base, H, p.n) < p.n) {
             T* const next = (T*)ring_smem + (buf ^ 1) * H;
             for (int k = threadIdx.x; k < H; k += blockDim.x) next[k] = Marker<T>::pending_value();
         }

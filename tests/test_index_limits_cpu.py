@@ -43,7 +43,25 @@ static void cursor(int lanes, int slots, int len, int longest) {
     }
 }
 
+// the windows of the last rows of a system of n rows: all of them, each once
+static void windows(int rows, int n) {
+    int base = n - n % rows - 3 * rows, seen = 0, count = 0;
+    if (base < 0) base = 0;
+    const int from = base;
+    for (; base < n; base = next_window(base, rows, n)) {
+        check(count == 0 || (base - from) % rows == 0, "window", base, n);
+        seen += n - base < rows ? n - base : rows;
+        if (++count > 5) break;
+    }
+    check(base == n && seen == n - from, "windows", base, seen);
+}
+
 int main() {
+    for (int rows : {12288, 24576})
+        for (int less : {0, 1, 255, 12287, 12288, 12289, 24576}) {
+            windows(rows, SPTRSV_MAX_SIZE - less);
+            windows(rows, less + 1);
+        }
     for (int lanes = 1; lanes <= 32; lanes *= 2)
         for (int len = 1; len <= 40; ++len) cursor(lanes, lanes >= 16 ? 2 : 4, len, 5000);
     return bad;
@@ -67,6 +85,11 @@ def answer(tmp_path_factory):
 
 def test_helpers_stay_inside_int(answer):
     assert answer.returncode == 0, answer.stdout + answer.stderr
+
+
+def test_windows_are_stepped_by_the_helper():
+    text = open(os.path.join(CSRC, "solve_cluster.cu")).read()
+    assert not re.search(r"base \+=|base \+ H", text)
 
 
 def test_chunks_of_a_warp_are_stepped_by_the_helper():
