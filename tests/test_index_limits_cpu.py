@@ -12,6 +12,7 @@ CSRC = os.path.join(ROOT, "paper_1710_04985_gb300", "csrc")
 
 PROGRAM = r"""
 #include <cstdio>
+#include <initializer_list>
 #include "cursor.h"
 #include "sptrsv.h"
 using namespace sptrsv;
