@@ -236,7 +236,8 @@ __device__ __forceinline__ bool mrhs_apart(const SolveParams& p, long long t, bo
 // tickets in hand already), the rows of the other tickets the warp holds must not
 // wait for it where they do not need it: turns of a few polls for all of them,
 // until they are done or the polls reach the spin limit, then one after the other
-// to its end.
+// to its end.  No ticket is taken ahead meanwhile: its rows would wait for that end,
+// and with them the rows of other warps that need them and not the missing value.
 template <typename T, int W, bool MAP, bool PERM>
 __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1, int h2,
                                            unsigned left, bool again) {
@@ -250,12 +251,15 @@ __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1,
         return t;  // in lane 0
     };
     long long polls = 0;
-    int slot = 0, tn = ticket();
+    int slot = 0, tn = 0;
+    bool ahead = false;  // tn is a ticket taken ahead
     while (true) {
         if (left == 0) {
+            if (!ahead) tn = ticket();
             h0 = __shfl_sync(FULL, tn, 0);
             if ((long long)h0 * R >= p.n) return;
             tn = ticket();  // consumed after this one
+            ahead = true;
             left = 1;
             slot = 0;
             again = false;
@@ -270,8 +274,8 @@ __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1,
             again = true;
             polls = 0;
             h1 = __shfl_sync(FULL, tn, 0);
+            ahead = false;
             if ((long long)h1 * R < p.n) left |= 2u;
-            tn = ticket();
         } else {
             polls += kTurn;
         }
