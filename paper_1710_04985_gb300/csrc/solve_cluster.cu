@@ -30,9 +30,12 @@
 //
 // A value that does not come within a quarter of the spin limit: the warp raises a
 // flag in every block, all warps leave their waits and meet at the barrier, and the
-// rows that are left are computed level by level, a barrier between two levels.
-// Nothing is waited for there: what is missing then never comes (it is reported and
-// taken as NaN), and every row that does not depend on it is exact.
+// rows that are left of the window are computed level by level, a barrier between two
+// levels.  Nothing is waited for there: what is missing then never comes (it is
+// reported and taken as NaN), and every row that does not depend on it is exact.  A
+// warp's groups are in level order, so it goes through them once.  The next window
+// runs as usual; a value of an earlier window that is missing there was never
+// published and is not waited for either.
 #include "self_rows.cuh"
 
 namespace sptrsv {
@@ -76,7 +79,7 @@ template <typename T, int W, bool MAP, bool PERM>
 __global__ void __launch_bounds__(kClusterBlock, 1)
     cluster_solve_k1(const __grid_constant__ SolveParams p, int nblocks) {
     extern __shared__ __align__(16) unsigned char ring_smem[];
-    __shared__ int s_bail[2];  // by parity of the window: read after its barrier
+    __shared__ int s_bail[2];  // by parity of the window: read after its barrier, then cleared
     constexpr int R = 32 / W;
     constexpr int E = ChunkOf<W>::E;
     constexpr int H = kWindowBytes / (int)sizeof(T);  // rows of a window, a multiple of 32
@@ -100,7 +103,6 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
     if (threadIdx.x < 2) s_bail[threadIdx.x] = 0;
     cluster_sync();
 
-    bool slow = false;
     int buf = 0;
     for (int base = 0; base < p.n; base = next_window(base, H, p.n), buf ^= 1) {
         const T* const ring = (const T*)ring_smem + buf * H;
@@ -137,7 +139,7 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
             T* const next = (T*)ring_smem + (buf ^ 1) * H;
             for (int k = threadIdx.x; k < H; k += blockDim.x) next[k] = Marker<T>::pending_value();
         }
-        for (int g = rank + nblocks * warp; !slow && g * R < rows; g += nblocks * nwarps) {
+        for (int g = rank + nblocks * warp; g * R < rows; g += nblocks * nwarps) {
             if (__any_sync(FULL, *bail != 0)) break;
             Row<T> r = take_row<T, W, PERM>(p, (long long)base + g * R + grp);
             start_row<T, W, MAP>(p, r, sl);
@@ -184,6 +186,13 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
                         if (__any_sync(FULL, act)) break;
                     }
                     if (++polls > kClusterHot) {
+#pragma unroll
+                        for (int e = 0; e < E; ++e)
+                            if (at[e] < 0 && Marker<T>::pending(v[e])) {
+                                // of an earlier window: it never comes
+                                report(p.status, r.i, kCodeTimeout);
+                                v[e] = Marker<T>::canonical_nan();
+                            }
                         if (polls > patience && lane < nblocks)
                             st_block(cluster_addr(smem_addr(&s_bail[buf]), lane), 1);
                         if (__any_sync(FULL, *bail != 0) || polls > 2 * patience + 1024) {
@@ -229,40 +238,46 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
         }
         __syncwarp();
         cluster_sync();
-        slow = slow || *bail;  // the same in every block
-        if (!slow) continue;
+        if (!*bail) continue;  // the same in every block
         // level by level: what has not been published by now and is not published
         // one barrier later never is
         const int last = p.lev[p.jlev[base + rows - 1]];
+        int g = rank + nblocks * warp;  // this warp's lowest group with rows left
         for (int m = p.lev[p.jlev[base]]; m <= last; ++m) {
-            for (int g = rank + nblocks * warp; g * R < rows; g += nblocks * nwarps) {
+            for (; g * R < rows; g += nblocks * nwarps) {
                 Row<T> r = take_row<T, W, PERM>(p, (long long)base + g * R + grp);
-                const bool act = r.has && p.lev[r.i] == m &&
+                const int lev = r.has ? p.lev[r.i] : m;
+                const bool act = r.has && lev == m &&
                                  Marker<T>::pending(lds_relaxed(ring + (r.k - base)));
-                if (!__any_sync(FULL, act)) continue;
-                start_row<T, W, MAP>(p, r, sl);
-                int c[E];
-                T a[E];
-                for (int q0 = r.beg + sl; __any_sync(FULL, act && q0 < r.end);
-                     q0 = advance(q0, W * E, r.end)) {
-                    load_entries<T, W, MAP, PERM, E>(p, r, q0, c, a);
-                    scale_entries(p, r.dinv, c, a);
+                if (__any_sync(FULL, act)) {
+                    start_row<T, W, MAP>(p, r, sl);
+                    int c[E];
+                    T a[E];
+                    for (int q0 = r.beg + sl; __any_sync(FULL, act && q0 < r.end);
+                         q0 = advance(q0, W * E, r.end)) {
+                        load_entries<T, W, MAP, PERM, E>(p, r, q0, c, a);
+                        scale_entries(p, r.dinv, c, a);
 #pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        if (act && c[e] >= 0) {
-                            T v = look(c[e], place(c[e]));
-                            if (Marker<T>::pending(v)) {
-                                report(p.status, r.i, kCodeTimeout);
-                                v = Marker<T>::canonical_nan();
+                        for (int e = 0; e < E; ++e)
+                            if (act && c[e] >= 0) {
+                                T v = look(c[e], place(c[e]));
+                                if (Marker<T>::pending(v)) {
+                                    report(p.status, r.i, kCodeTimeout);
+                                    v = Marker<T>::canonical_nan();
+                                }
+                                r.sum = fma(-a[e], v, r.sum);
                             }
-                            r.sum = fma(-a[e], v, r.sum);
-                        }
+                    }
+                    publish(r, act, row_sum<W>(r.sum, warp_span<W>(r.has, r.end - r.beg)));
                 }
-                publish(r, act, row_sum<W>(r.sum, warp_span<W>(r.has, r.end - r.beg)));
+                if (__any_sync(FULL, lev > m)) break;  // rows of a later level
             }
             __syncwarp();
             cluster_sync();
         }
+        // every thread has read the flag by now, and the next window of this parity
+        // begins two barriers from here
+        if (threadIdx.x == 0) *bail = 0;
     }
 }
 
