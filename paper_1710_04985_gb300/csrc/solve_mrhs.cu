@@ -124,7 +124,8 @@ __device__ __forceinline__ void publish_column(const SolveParams& p, T* at, int 
 // The rows of ticket t, every lane at its own pace: a column is folded as its
 // values come and published by itself.  Gives up (false) after `budget` polls
 // without an end; again: columns that are published already are skipped.
-template <typename T, int W, bool MAP, bool PERM>
+// ONE: one count of polls for both ends, the budget and the spin limit.
+template <typename T, int W, bool MAP, bool PERM, bool ONE>
 __device__ __forceinline__ bool mrhs_apart(const SolveParams& p, long long t, bool again,
                                         long long budget) {
     constexpr unsigned FULL = 0xffffffffu;
@@ -187,6 +188,7 @@ __device__ __forceinline__ bool mrhs_apart(const SolveParams& p, long long t, bo
     };
     if (!lane_done) start_column();
     if (!lane_done) adopt_chunk();
+    const long long stop = budget < p.spin.limit ? budget + 1 : p.spin.limit;
     long long waits = 0, total = 0;
     unsigned ns = 32;
     while (true) {
@@ -210,8 +212,9 @@ __device__ __forceinline__ bool mrhs_apart(const SolveParams& p, long long t, bo
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 if ((pend & (1u << e)) && !Marker<T>::pending(v[e])) pend &= ~(1u << e);
-            if (++total > budget) return false;
-            if (++waits >= p.spin.limit) {
+            if (!ONE && ++total > budget) return false;
+            if (++waits >= (ONE ? stop : p.spin.limit)) {
+                if (ONE && waits > budget) return false;
                 if (pend) {
                     report(p.status, i, kCodeTimeout);
 #pragma unroll
@@ -238,7 +241,7 @@ __device__ __forceinline__ bool mrhs_apart(const SolveParams& p, long long t, bo
 // until they are done or the polls reach the spin limit, then one after the other
 // to its end.  No ticket is taken ahead meanwhile: its rows would wait for that end,
 // and with them the rows of other warps that need them and not the missing value.
-template <typename T, int W, bool MAP, bool PERM>
+template <typename T, int W, bool MAP, bool PERM, bool ONE>
 __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1, int h2,
                                            unsigned left, bool again) {
     constexpr unsigned FULL = 0xffffffffu;
@@ -251,15 +254,13 @@ __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1,
         return t;  // in lane 0
     };
     long long polls = 0;
-    int slot = 0, tn = 0;
-    bool ahead = false;  // tn is a ticket taken ahead
+    int slot = 0, tn = -1;  // no ticket taken ahead
     while (true) {
         if (left == 0) {
-            if (!ahead) tn = ticket();
             h0 = __shfl_sync(FULL, tn, 0);
-            if ((long long)h0 * R >= p.n) return;
             tn = ticket();  // consumed after this one
-            ahead = true;
+            if (h0 < 0) continue;
+            if ((long long)h0 * R >= p.n) return;
             left = 1;
             slot = 0;
             again = false;
@@ -268,13 +269,13 @@ __device__ __forceinline__ void apart_rest(const SolveParams& p, int h0, int h1,
         const int t = slot == 0 ? h0 : slot == 1 ? h1 : h2;
         const long long budget = !again                  ? p.spin.limit / 4 + 1
                                  : polls < p.spin.limit ? kTurn : kNoEnd;
-        if (mrhs_apart<T, W, MAP, PERM>(p, t, again, budget)) {
+        if (mrhs_apart<T, W, MAP, PERM, ONE>(p, t, again, budget)) {
             left &= ~(1u << slot);
         } else if (!again) {  // stuck: the ticket ahead takes turns with this one
             again = true;
             polls = 0;
             h1 = __shfl_sync(FULL, tn, 0);
-            ahead = false;
+            tn = -1;
             if ((long long)h1 * R < p.n) left |= 2u;
         } else {
             polls += kTurn;
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(1024) level_mrhs_k(const __grid_constant__ Sol
 template <typename T, int W, bool MAP, bool PERM>
 __global__ void __launch_bounds__(kMaxMrhsBlock)
     apart_mrhs_k(const __grid_constant__ SolveParams p) {
-    apart_rest<T, W, MAP, PERM>(p, 0, 0, 0, 0, false);
+    apart_rest<T, W, MAP, PERM, true>(p, 0, 0, 0, 0, false);
 }
 
 // Rows that are alike.  MULTI: rows of more than one chunk of entries.
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(kMaxMrhsBlock, 3)
         }
         const int t2 = __shfl_sync(FULL, tn, 0);
         if (!ok) {
-            apart_rest<T, W, MAP, PERM>(p, t, t1, t2,
+            apart_rest<T, W, MAP, PERM, false>(p, t, t1, t2,
                                         1u | ((long long)t1 * R < p.n ? 2u : 0u) |
                                             ((long long)t2 * R < p.n ? 4u : 0u), true);
             return;
