@@ -828,24 +828,55 @@ int max_part_rows(sptrsv_plan_t P) {
     return room > esize * 32 ? (room / esize) & ~31 : 32;
 }
 
-// Whether the rows of every ticket of the self-scheduled kernel are taken as one:
-// rows of about equal length, and tickets of 32 / lanes rows that span few
-// levels on average.  (In-place solves before and after, us: 7-point 128^3 570 ->
-// 514, 27-point 61 x 47 x 53 467 -> 380, 5-point 120 x 130 249 -> 239.)
-bool rows_alike(sptrsv_plan_t P, const Levels& L, int lanes) {
-    return (long long)L.max_len * P->n <= 2ll * P->nnz + 2ll * P->n &&
+// Entries of the longest row beside the diagonal.
+int row_entries(sptrsv_plan_t P, const Levels& L) { return L.max_len - (P->unit ? 0 : 1); }
+
+// Rows of about equal length, and such rows in tickets (32 / lanes rows) that span few
+// levels on average.
+bool lengths_like(sptrsv_plan_t P, const Levels& L) {
+    return (long long)L.max_len * P->n <= 2ll * P->nnz + 2ll * P->n;
+}
+bool rows_like(sptrsv_plan_t P, const Levels& L, int lanes) {
+    return lengths_like(P, L) &&
            32ll * L.nlev <= 3ll * lanes * P->n;
+}
+
+// Whether the rows of every ticket of a self-scheduled kernel are taken as one: like
+// rows, and where a ticket straddles levels they are one chunk of entries, or such
+// tickets are rare (levels of at least four tickets).  A ticket of two levels is gone
+// through level by level: rows of one chunk hold theirs in registers, but a longer row
+// of the second level would begin when the first level is done, so that all its chunks
+// come after one another on the chain.  (In-place solves rows apart and as one, us:
+// 7-point 128^3 570 and 514, 27-point 61 x 47 x 53 467 and 380, 5-point 120 x 130 249
+// and 239; but the dense triangle of 2000 rows with 8 lanes 1660 and 38900, its solve
+// for 16 columns 1730 and 207000, a band of 40 for 16 columns 26500 and 96100.)
+bool rows_alike(sptrsv_plan_t P, const Levels& L, int lanes, int chunk) {
+    return rows_like(P, L, lanes) &&
+           (lanes == 32 || row_entries(P, L) <= chunk ||
+            128ll * L.nlev <= (long long)lanes * P->n);
+}
+// Entries of a row that a kernel for one right-hand side takes at once (self_rows.cuh).
+int row_chunk(int lanes) { return lanes * (lanes >= 16 ? 2 : kChunk); }
+
+// Whether tickets span four levels and more on average.
+bool deep(sptrsv_plan_t P, const Levels& L, int lanes) {
+    return 8ll * L.nlev >= (long long)P->n * lanes;
 }
 
 // Whether a single-RHS solve of the in-place or level-ordered form runs in one
 // block with its unknowns in shared memory: they must fit there, rows must be
-// alike, and an average level must hold few enough row groups (32 / lanes rows)
-// for one SM.  (5-point grids, plan defaults, us: 64 x 64 FP64 123 -> 82 and FP32
+// like one another, and an average level must hold few enough row groups (32 / lanes
+// rows) for one SM.  (5-point grids, plan defaults, us: 64 x 64 FP64 123 -> 82 and FP32
 // 115 -> 56 at two groups per level; 120 x 130 FP64 249 -> 196 at four; 160 x 160
 // FP32 299 -> 194 at five.  The 7-point 20 x 18 x 22 grid, 17 groups per level:
-// 71 us on the whole GPU, 170 in one block.)
+// 71 us on the whole GPU, 170 in one block.)  Rows are taken as one there, so those of
+// several chunks must not straddle levels much (rows_alike): one row per ticket, or two
+// chunks in tickets of few levels (band of 40, 20000 rows, FP64: 16 lanes and two levels
+// a ticket 13.9 ms, 18.4 on the whole GPU; 8 lanes and four levels 23.9 and 15.1).
 bool small_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes) {
-    if ((f64 ? 8ll : 4ll) * P->n > P->smem_optin - 128 || !rows_alike(P, L, lanes)) return false;
+    if ((f64 ? 8ll : 4ll) * P->n > P->smem_optin - 128 || !rows_like(P, L, lanes)) return false;
+    const int chunks = lanes == 32 ? L.max_len : deep(P, L, lanes) ? 1 : 2;
+    if (row_entries(P, L) > (long long)chunks * row_chunk(lanes)) return false;
     // FP32 rows take half the time: no FP64 unit to wait for
     return (long long)P->n * lanes <= 32ll * kSmallGroups * (f64 ? 1 : 2) * L.nlev;
 }
@@ -1212,7 +1243,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     const int a = (int)algo;
     const bool own = !mrhs && a >= 0 && a < 8 && P->alg_lanes[a] > 0;
     const int lanes = mrhs ? (P->mrhs_lanes ? P->mrhs_lanes
-                                            : mrhs_lanes(nrhs, per_level, rows_alike(P, Lt, 8)))
+                                            : mrhs_lanes(nrhs, per_level, rows_alike(P, Lt, 8, kChunk)))
                            : (own ? P->alg_lanes[a] : P->lanes);
     const int block = mrhs ? (P->mrhs_block ? P->mrhs_block : P->block)
                            : (own ? P->alg_block[a] : P->block);
@@ -1280,10 +1311,13 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     p.unit = P->unit;
     p.jlev = L.jlev;
     p.lev = L.lev;
-    p.rows_alike = rows_alike(P, L, lanes) ? 1 : 0;
+    // (one block takes them so too, small_solve)
+    const bool one_block = !mrhs && (algo == SPTRSV_ALGO_SELF || (permuted && !blocked)) &&
+                           small_solve(P, L, f64, lanes);
+    p.rows_alike = one_block || rows_alike(P, L, lanes, mrhs ? kChunk : row_chunk(lanes));
     // a unit diagonal need not be stored: then max_len counts no diagonal
     const MrhsRows mrows = !p.rows_alike ? kMrhsApart
-                           : L.max_len - (P->unit ? 0 : 1) <= kChunk ? kMrhsShort : kMrhsAlike;
+                           : row_entries(P, L) <= kChunk ? kMrhsShort : kMrhsAlike;
     p.b = b;
     p.ldb = ldb;
     p.x = x;
@@ -1401,16 +1435,15 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         p.vals = f32_of_f64 ? L.pvals32 : L.pvals;
         p.xp = f32_of_f64 ? L.xp32 : L.xp;
         p.prescaled = P->unit ? 0 : 1;
-        const bool small = !blocked && small_solve(P, L, f64, lanes);
         const int on_cluster =
-            blocked || small ? 0 : cluster_solve(P, L, f64, lanes, max_blocks, false, true);
-        if (!small && !on_cluster)
+            blocked || one_block ? 0 : cluster_solve(P, L, f64, lanes, max_blocks, false, true);
+        if (!one_block && !on_cluster)
             CK(launch_prep_self(f64, P->n, 1, p.xp, 1, nullptr, 0, nullptr, P->counters,
                                 P->num_sms * 8, s));
         const int R = 32 / lanes;
         const long long tickets = ((long long)P->n + R - 1) / R;
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
-        if (small) {
+        if (one_block) {
             ST(prof_begin(P, s));
             CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
             ST(prof_end(P, s));
@@ -1437,8 +1470,8 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             CK(launch_self_k1(f64, lanes, p, (int)grid, block, s));
             ST(prof_end(P, s));
         }
-        launches = small || on_cluster ? 1 : 2;
-    } else if (algo == SPTRSV_ALGO_SELF && !mrhs && small_solve(P, L, f64, lanes)) {
+        launches = one_block || on_cluster ? 1 : 2;
+    } else if (one_block) {
         ST(prof_begin(P, s));
         CK(launch_self_small(f64, lanes, p, kSmallBlock, s));
         ST(prof_end(P, s));

@@ -83,7 +83,9 @@ constexpr int kSelfHot = 64;        // polls of one wait before the warp backs o
 // Whether the warp takes the rows of a ticket as one, where the matrix as a
 // whole does not say so (SolveParams::rows_alike): equally many chunks of
 // entries, lengths within a factor of about two (unless there are only two
-// rows), and at most kLevels levels.  A general matrix of 20001 rows with 4 lanes
+// rows), and one level, or at most kLevels levels of rows of one chunk (longer rows of
+// its second level would begin when the first is done: dense triangle of 2000 rows, 8
+// lanes, 38.9 ms as one and 1.7 apart).  A general matrix of 20001 rows with 4 lanes
 // per row (mean row 14 entries, longest 900) took 2.36 ms with every ticket as
 // one and 1.09 ms with its rows apart.
 template <int W>
@@ -94,8 +96,8 @@ __device__ __forceinline__ bool alike(bool has, int len, int lev) {
     const int least = __reduce_min_sync(FULL, has ? len : 0x7fffffff);
     const int top = __reduce_max_sync(FULL, has ? lev : -1);
     const int low = __reduce_min_sync(FULL, has ? lev : 0x7fffffff);
-    if (top - low >= kLevels) return false;
     constexpr int C = W * ChunkOf<W>::E;
+    if (top - low >= (most > C ? 1 : kLevels)) return false;
     if ((most + C - 1) / C != (least + C - 1) / C) return false;
     return W >= 16 || most <= 2 * least + 2;
 }
