@@ -18,7 +18,8 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 INCLUDE = os.path.join(ROOT, "include")
 
-SOURCES = ["api.cu", "analysis.cu", "solve_self.cu", "solve_cluster.cu", "solve_level.cu", "solve_mrhs.cu", "aux.cu",
+SOURCES = ["api.cu", "analysis.cu", "solve_self.cu", "solve_apart.cu", "solve_cluster.cu",
+           "solve_level.cu", "solve_mrhs.cu", "aux.cu",
            "solve_tiled.cu", "solve_chain.cu", "noalloc.cu", "permute.cu",
            "solve_column.cu", "kahn.cu", "solve_blocked.cu", "solve_parts.cu",
            "solve_partitioned_f64.cu", "solve_partitioned_f32.cu", "refine.cu"]

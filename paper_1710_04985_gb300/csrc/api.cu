@@ -881,6 +881,43 @@ bool small_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes) {
     return (long long)P->n * lanes <= 32ll * kSmallGroups * (f64 ? 1 : 2) * L.nlev;
 }
 
+// Tickets of an average level.
+double level_tickets(sptrsv_plan_t P, const Levels& L, int lanes) {
+    return (double)P->n * lanes / (32.0 * (L.nlev > 0 ? L.nlev : 1));
+}
+
+// Whether a single-RHS solve of the in-place or level-ordered form on the whole GPU
+// takes every row at its own pace (solve_apart.cu) instead of asking for tickets whose
+// rows are alike (solve_self.cu).  Measured on 18 matrices, both types, all widths, as
+// the time with the second over the time with the first:
+//  * Levels of more than kFlatLevel tickets: with up to 8 lanes 1.02 to 1.17, up to 1.5
+//    where the grid is not capped; with 16 lanes 0.97 to 1.1 and up to 1.5, with 32 lanes
+//    0.9 to 0.98 and up to 1.35.  Uncapped FP64 grids with 16 and 32 lanes cross
+//    earlier: 0.68 at 512 tickets, 1.03 (adjoint 1.14) at 1550, 1.09 at 3100.
+//  * Alike rows: only one lane in place and rows of up to three entries (5-point 1.1 to
+//    1.2, 7-point 1.05, 9-point 0.71; from two lanes on 0.6 to 0.95).
+//  * Rows that differ in tickets that span four levels and more on average, where asking
+//    is in vain: up to 4 lanes 1.07 to 1.22; 8 lanes FP64 1.03 to 1.5, FP32 0.87 for a
+//    chain and 1.2 for a band of 40.
+//  * Other rows that differ: adjoint up to 4 lanes 1.05 to 1.28, 8 lanes 0.95 and FP32
+//    0.86; in place up to 2 lanes 0.96 to 1.05, 4 lanes 1.04, 8 lanes 1.04 and FP32 0.96;
+//    level-ordered FP32 up to 4 lanes 1.02 to 1.05, FP64 0.87 to 1.0.  16 lanes 0.7 to
+//    0.85 throughout.
+constexpr double kFlatLevel = 8192.0;
+bool apart_solve(sptrsv_plan_t P, const Levels& L, bool f64, int lanes, int max_blocks, bool map,
+                 bool perm) {
+    const double tickets = level_tickets(P, L, lanes);
+    const int len = row_entries(P, L);
+    if (tickets > kFlatLevel) return lanes <= 16 || max_blocks == 0;
+    if (f64 && max_blocks == 0 && lanes >= 16 && tickets > kFlatLevel / 8) return true;
+    if (rows_alike(P, L, lanes, row_chunk(lanes))) return lanes == 1 && !perm && len < kChunk;
+    if (deep(P, L, lanes))
+        return lanes <= 4 || (lanes == 8 && (f64 || len > row_chunk(lanes)));
+    if (perm) return lanes <= 4 && !f64;
+    if (map) return lanes <= 4;
+    return lanes == 4 || (lanes == 8 && f64);
+}
+
 // Blocks of the cluster that a single-RHS solve of the in-place or level-ordered
 // form runs on, 0: the whole GPU.  On a cluster a hop is shorter, but every row is
 // stored into each of its blocks and 16 SMs fold: an average level must hold at most
@@ -1220,6 +1257,31 @@ sptrsv_status_t prof_end(sptrsv_plan_t P, cudaStream_t s) {
     return SPTRSV_OK;
 }
 
+// A single-RHS solve of the in-place or level-ordered form (p.xp) on the whole GPU.
+sptrsv_status_t launch_whole(sptrsv_plan_t P, const Levels& L, bool f64, int lanes,
+                             const SolveParams& p, int block, int max_blocks,
+                             long long want_blocks, cudaStream_t s) {
+    const bool perm = p.xp != nullptr, map = !perm && p.vmap;
+    const bool apart = apart_solve(P, L, f64, lanes, max_blocks, map, perm);
+    long long per_sm = apart ? apart_blocks_per_sm(f64, lanes, map, perm, block)
+                             : self_k1_blocks_per_sm(f64, lanes, map, perm, block);
+    // Unless levels are very wide, more than 512 threads an SM only flood L2 with polls
+    // (general 100001 rows, 2 lanes, FP64: 2048 threads 21.8 ms, 512 threads 12.4).
+    if (apart && level_tickets(P, L, lanes) <= kFlatLevel / 8) {
+        const int most = block < 512 ? 512 / block : 1;
+        if (per_sm > most) per_sm = most;
+    }
+    long long grid = per_sm * P->num_sms;
+    if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
+    if (grid > want_blocks) grid = want_blocks;
+    if (grid < 1) grid = 1;
+    ST(prof_begin(P, s));
+    CK(apart ? launch_apart_k1(f64, lanes, p, (int)grid, block, s)
+             : launch_self_k1(f64, lanes, p, (int)grid, block, s));
+    ST(prof_end(P, s));
+    return SPTRSV_OK;
+}
+
 // One triangular solve (forward pattern or transpose) of any element type:
 // `f64` selects the kernels, `vals` the values they read.
 // Whether a solve of this form can accumulate its published values into an
@@ -1461,14 +1523,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             CK(launch_blocked_k1(f64, lanes, p, P->tile_rows, (int)grid, block, s));
             ST(prof_end(P, s));
         } else {
-            long long grid =
-                (long long)self_k1_blocks_per_sm(f64, lanes, false, true, block) * P->num_sms;
-            if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
-            if (grid > want_blocks) grid = want_blocks;
-            if (grid < 1) grid = 1;
-            ST(prof_begin(P, s));
-            CK(launch_self_k1(f64, lanes, p, (int)grid, block, s));
-            ST(prof_end(P, s));
+            ST(launch_whole(P, L, f64, lanes, p, block, max_blocks, want_blocks, s));
         }
         launches = one_block || on_cluster ? 1 : 2;
     } else if (one_block) {
@@ -1499,9 +1554,9 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
         const int R = 32 / lanes;
         const long long tickets = ((long long)P->n + R - 1) / R;
         const long long want_blocks = (tickets + block / 32 - 1) / (block / 32);
-        long long grid = P->num_sms *
-                         (long long)(mrhs ? mrhs_blocks_per_sm(f64, lanes, trans, false, mrows, block)
-                                          : self_k1_blocks_per_sm(f64, lanes, trans, false, block));
+        long long grid =
+            mrhs ? (long long)mrhs_blocks_per_sm(f64, lanes, trans, false, mrows, block) * P->num_sms
+                 : want_blocks;
         if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
         if (grid > want_blocks) grid = want_blocks;
         if (grid < 1) grid = 1;
@@ -1525,10 +1580,13 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
                                s));
             ST(prof_end(P, s));
         } else {
-            ST(prof_begin(P, s));
-            CK(mrhs ? launch_mrhs(f64, lanes, true, mrows, p, (int)grid, block, s)
-                    : launch_self_k1(f64, lanes, p, (int)grid, block, s));
-            ST(prof_end(P, s));
+            if (mrhs) {
+                ST(prof_begin(P, s));
+                CK(launch_mrhs(f64, lanes, true, mrows, p, (int)grid, block, s));
+                ST(prof_end(P, s));
+            } else {
+                ST(launch_whole(P, L, f64, lanes, p, block, max_blocks, want_blocks, s));
+            }
         }
         launches = 2;
     }

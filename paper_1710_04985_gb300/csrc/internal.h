@@ -142,6 +142,10 @@ cudaError_t launch_part_k1(bool f64, int lanes, const SolveParams& p, int grid, 
 int part_resident_blocks(bool f64, int lanes, int cluster, int block, int part_rows, int num_sms);
 // Resident blocks per SM of self_solve_k1 (perm: its level-ordered-copy form).
 int self_k1_blocks_per_sm(bool f64, int lanes, bool map, bool perm, int block);
+// The kernel that takes every row at its own pace (solve_apart.cu), same arguments.
+cudaError_t launch_apart_k1(bool f64, int lanes, const SolveParams& p, int grid, int block,
+                            cudaStream_t s);
+int apart_blocks_per_sm(bool f64, int lanes, bool map, bool perm, int block);
 // The whole system in one block, its unknowns in shared memory (n * element size
 // at most the device's opt-in shared memory per block, minus 128 B).  Needs no
 // prep launch: b is read before x is written, in place too.
