@@ -76,11 +76,12 @@ struct Levels {
     int* qrow = nullptr;
     int qnparts = 0, qmaxpart = 0, qnblocks = 0;
     // Sliced copy of the matrix in part order, per log2(lanes) (built on first
-    // use; layout in solve_parts.cu).  wide: its padding would take more than
-    // kMaxPadding times the stored entries, so it is not built and solves of
-    // this width run on the level-ordered copy.
+    // use; layout in solve_parts.cu).  form: what partitioned solves of this width
+    // run on (slice_form); only kSliced has a copy.
+    enum Form { kSliced, kLevelOrder, kInPlace };
     struct Slices {
-        bool built = false, wide = false;
+        bool built = false;
+        Form form = kSliced;
         int ngroups = 0;
         long long slots = 0;
         int4* grp = nullptr;
@@ -105,8 +106,6 @@ struct Levels {
 };
 
 // Sliced copies larger than this many times the stored entries are not built.
-// Each slot costs a load in the solve; a width at which eight in nine slots are
-// empty is never the one to use.
 constexpr long long kMaxPadding = 8;
 constexpr int kSmallBlock = 512;  // threads of a solve in one block, and
 constexpr int kSmallGroups = 4;   // the row groups per level it is used for
@@ -1090,6 +1089,35 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     return SPTRSV_OK;
 }
 
+// What partitioned solves of one width run on: the sliced copy, unless
+//  * a warp would go through many chunks of slots one after another.  It holds one group
+//    of one level, so in parts of narrow levels few rows are on their way, and long rows
+//    among them wait for their turn: extra chunks of earlier parts' slots, per 32/lanes
+//    rows, above 1.25 where lengths differ, above 16 where they do not, or above 64 of
+//    the part's own.  Times over those of the blocked kernel on a part-ordered CSR copy
+//    that served this form before: general matrices 0.5 to 0.7 up to 1.3, 0.8 to 1.3 at
+//    1.4, 0.6 to 1.7 at 2 to 8, 1.1 to 2.8 above, where the level-ordered copy takes 0.5
+//    to 0.9 all along; 27-point grids 0.3 to 0.6 up to 15; the dense triangle of 2000 rows
+//    0.65 at 15 and 1.9 to 12 from 60 on; own slots of a band of 40 0.5 at 17 and of the
+//    dense triangle 1.2 to 2 from 120 on;
+//  * more than seven in eight slots would be empty (kMaxPadding): with 32 lanes in place
+//    (5-point 1024 x 1024, FP64: 1.72 ms, level-ordered 2.35, the kernel before 1.87),
+//    else level-ordered (band of 40, one lane: 28.1 ms, in place 32.5);
+//  * levels are wide (more than 512 tickets), so that the empty slots count, and nearly
+//    half of them are empty (7-point 96^3, 16 lanes: 0.97 ms, level-ordered 0.54).
+// All three give bitwise the same result.
+Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long slots,
+                        const unsigned long long* more) {
+    const double rows = (double)P->n * lanes / 32.0;  // groups if all were full
+    if ((double)more[0] > (lengths_like(P, L) ? 16.0 : 1.25) * rows || (double)more[1] > 64.0 * rows)
+        return Levels::kLevelOrder;
+    if (slots > kMaxPadding * P->nnz + (1 << 20))
+        return lanes == 32 ? Levels::kInPlace : Levels::kLevelOrder;
+    if (4 * slots > 7ll * P->nnz && level_tickets(P, L, lanes) > 512.0)
+        return Levels::kLevelOrder;
+    return Levels::kSliced;
+}
+
 // Sliced copy of one direction's matrix in part order (which must exist) for
 // one sub-warp width: the row groups (runs of equal level inside a part, cut
 // into groups of at most 32/lanes rows), their shapes, columns and values,
@@ -1106,8 +1134,10 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     Levels::Slices q;
     int* scratch = nullptr;
     int h[2] = {0, 0};  // groups, slices
-    cudaError_t e = cudaMalloc(&scratch, sizeof(int) * (5 * N + 5));
-    int* flag = scratch;           // of the runs; then the group starts
+    unsigned long long h_more[2] = {0, 0};
+    cudaError_t e = cudaMalloc(&scratch, sizeof(int) * (5 * N + 9));
+    unsigned long long* more = (unsigned long long*)scratch;
+    int* flag = scratch + 4;       // of the runs; then the group starts
     int* scan = flag + (N + 1);    // of the run flags, then of the group flags
     int* rstart = scan + (N + 1);  // run starts; then the groups' slice counts
     int* gflag = rstart + (N + 1);
@@ -1129,18 +1159,21 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     const int *gstart = flag, *cnt = rstart;
     if (e == cudaSuccess) e = cudaMalloc(&q.grp, sizeof(int4) * (size_t)q.ngroups);
     const SliceParams sp = slice_params(P, trans, q);
-    if (e == cudaSuccess) e = launch_group_shapes(sp, lanes, gstart, q.grp, rstart, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(more, 0, sizeof(h_more), s);
+    if (e == cudaSuccess) e = launch_group_shapes(sp, lanes, gstart, q.grp, rstart, more, s);
     if (e == cudaSuccess) e = launch_exclusive_scan(cnt, base, q.ngroups, P->scan_sums, s);
     if (e == cudaSuccess) e = launch_group_bases(q.ngroups, base, q.grp, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&h[1], base + q.ngroups, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h_more, more, sizeof(h_more), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     // a lane holds at most its rows' entries, so the slices are at most nnz
     if (e == cudaSuccess && (h[1] < 0 || h[1] > P->nnz)) e = cudaErrorUnknown;
     q.slots = 32ll * h[1];
-    q.wide = q.slots > kMaxPadding * P->nnz + (1 << 20);
+    if (e == cudaSuccess) q.form = slice_form(P, L, lanes, q.slots, h_more);
     const size_t slots = q.slots > 0 ? (size_t)q.slots : 1;
-    if (e == cudaSuccess && !q.wide) {
+    if (e == cudaSuccess && q.form == Levels::kSliced) {
         e = cudaMalloc(&q.cols, sizeof(int) * slots);
         if (e == cudaSuccess) e = cudaMalloc(&q.vals, esize * slots);
         if (e == cudaSuccess && !P->unit) e = cudaMalloc(&q.dinv, esize * N);
@@ -1151,11 +1184,11 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
             cudaFree(q.vals);
             q.cols = nullptr;
             q.vals = nullptr;
-            q.wide = true;
+            q.form = Levels::kLevelOrder;
             e = cudaSuccess;
         }
     }
-    if (e == cudaSuccess && !q.wide) {
+    if (e == cudaSuccess && q.form == Levels::kSliced) {
         if (e == cudaSuccess)
             e = launch_fill_slices(P->f64, sp, lanes, q.grp, P->vals, q.cols, q.vals, q.dinv, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1168,6 +1201,11 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     if (rc != SPTRSV_OK) {
         free_slices(q);
         return rc;
+    }
+    if (q.form != Levels::kSliced) {  // nothing reads the groups
+        const Levels::Form form = q.form;
+        free_slices(q);
+        q.form = form;
     }
     q.built = true;
     L.qs[w] = q;
@@ -1322,26 +1360,27 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     if (parts) {
         ST(build_parts(P, trans, s));
         // While s is being captured a copy cannot be built for another width than
-        // the one prepared: that solve runs in place (bitwise the same result),
-        // with the publication buffer of the parts to keep b in.
+        // the one prepared: that solve runs in place (bitwise the same result).
         const Levels& Lq = trans ? P->trn : P->fwd;
         const Levels::Slices& q = Lq.qs[log2_lanes(lanes)];
-        if (!f32_of_f64 && (!q.built || (q.wide && !Lq.pptr)) && capturing(s))
-            for (const Levels::Slices& o : Lq.qs)
-                if (o.built) stand_in = Lq.xq;
-        if (stand_in) {
+        bool in_place = false;
+        if (!f32_of_f64 && capturing(s) &&
+            (!q.built || (q.form == Levels::kLevelOrder && !Lq.pptr)))
+            for (const Levels::Slices& o : Lq.qs) in_place = in_place || o.built;
+        if (!in_place) {
+            ST(build_slices(P, trans, lanes, s));
+            in_place = q.form == Levels::kInPlace;
+            parts = q.form == Levels::kSliced;
+            if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
+        }
+        if (in_place) {
+            stand_in = Lq.xq;  // the publication buffer of the parts holds b
             algo = SPTRSV_ALGO_SELF;
             parts = false;
         }
     }
-    if (parts) {
-        ST(build_slices(P, trans, lanes, s));
-        parts = !(trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].wide;
-        if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
-    }
     const bool blocked = algo == SPTRSV_ALGO_SELF_BLOCKED && !mrhs;
-    // a partitioned solve whose sliced copy would be mostly padding runs on the
-    // level-ordered copy (bitwise the same result)
+    // (a partitioned solve for which slice_form chose the level-ordered copy too)
     const bool permuted = (algo == SPTRSV_ALGO_SELF_PERMUTED || blocked ||
                            (algo == SPTRSV_ALGO_SELF_PARTITIONED && !parts)) && !mrhs;
     if (permuted) ST(build_permuted(P, trans, s));
@@ -1829,7 +1868,7 @@ sptrsv_status_t sptrsv_prepare(sptrsv_plan_t plan, int transpose, sptrsv_algo_t 
         case SPTRSV_ALGO_SELF_PARTITIONED:
             ST(build_parts(P, trans, s));
             ST(build_slices(P, trans, lanes, s));
-            if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].wide)
+            if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].form == Levels::kLevelOrder)
                 ST(build_permuted(P, trans, s));
             break;
         case SPTRSV_ALGO_SELF_COLUMN: ST(build_column(P, trans, s)); break;

@@ -221,10 +221,14 @@ struct SliceParams {
     int ngroups;
     unsigned long long* status;
 };
+// Slots of a group that the partitioned kernel takes at once: of earlier parts' entries
+// and of the part's own.
+constexpr int kExtChunk = 2, kOwnChunk = 4;
 // Descriptor of every group (its base left 0) from the group starts gstart
-// (ngroups + 1), and the number of its slices.
+// (ngroups + 1), and the number of its slices.  more (two zeros): chunks beyond the
+// first, of earlier parts' slots and of the part's own, over all groups.
 cudaError_t launch_group_shapes(const SliceParams& p, int lanes, const int* gstart, int4* grp,
-                                int* nslices, cudaStream_t s);
+                                int* nslices, unsigned long long* more, cudaStream_t s);
 // grp[g].y = base[g].
 cudaError_t launch_group_bases(int ngroups, const int* base, int4* grp, cudaStream_t s);
 // Slices of every group: columns (nullptr: values only), values and 1/d(i)

@@ -340,8 +340,8 @@ __global__ void __launch_bounds__(kMaxBlock, 1) part_solve_k1(const __grid_const
     T* xs = (T*)part_smem;
     __shared__ int s_part;
     __shared__ int s_pst[kMaxCluster];
-    constexpr int NI = 4;  // own-part slots, and
-    constexpr int NX = 2;  // earlier-part slots of a group loaded ahead
+    constexpr int NI = kOwnChunk;  // own-part slots, and
+    constexpr int NX = kExtChunk;  // earlier-part slots of a group loaded ahead
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;

@@ -272,10 +272,16 @@ __device__ __forceinline__ FoldRow fold_row(const SliceParams& p, int k, bool ha
     return r;
 }
 
+// more[0] and more[1] add up the chunks of every group beyond its first, of earlier
+// parts' slots and of the part's own.
 template <int W>
 __global__ void group_shapes_k(SliceParams p, const int* __restrict__ gstart, int4* grp,
-                               int* nslices) {
+                               int* nslices, unsigned long long* more) {
     constexpr unsigned FULL = 0xffffffffu;
+    __shared__ unsigned long long s_more[2];
+    if (threadIdx.x < 2) s_more[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long more_x = 0, more_i = 0;
     const int lane = threadIdx.x & 31, grow = lane / W, sl = lane % W;
     const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < p.ngroups;
@@ -299,8 +305,16 @@ __global__ void group_shapes_k(SliceParams p, const int* __restrict__ gstart, in
         if (lane == 0) {
             grp[g] = make_int4(k0, 0, X, (I << 12) | (span << 6) | cnt);
             nslices[g] = X + I;
+            if (X > kExtChunk) more_x += (X - 1) / kExtChunk;
+            if (I > kOwnChunk) more_i += (I - 1) / kOwnChunk;
         }
     }
+    if (lane == 0) {
+        if (more_x) atomicAdd(s_more, more_x);
+        if (more_i) atomicAdd(s_more + 1, more_i);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 && s_more[threadIdx.x]) atomicAdd(more + threadIdx.x, s_more[threadIdx.x]);
 }
 
 __global__ void group_bases_k(int ngroups, const int* __restrict__ base, int4* grp) {
@@ -466,9 +480,9 @@ static int warps_grid(long long warps) {  // 8 warps a block
 }
 
 cudaError_t launch_group_shapes(const SliceParams& p, int lanes, const int* gstart, int4* grp,
-                                int* nslices, cudaStream_t s) {
+                                int* nslices, unsigned long long* more, cudaStream_t s) {
     const int g = warps_grid(p.ngroups);
-#define SPTRSV_SHAPES(W) group_shapes_k<W><<<g, 256, 0, s>>>(p, gstart, grp, nslices)
+#define SPTRSV_SHAPES(W) group_shapes_k<W><<<g, 256, 0, s>>>(p, gstart, grp, nslices, more)
     switch (lanes) {
         case 1: SPTRSV_SHAPES(1); break;
         case 2: SPTRSV_SHAPES(2); break;

@@ -56,3 +56,50 @@ def test_tickets_of_long_rows_that_straddle_levels(make, algo):
             assert _ms(lambda: p.solve(one, algo=algo)) < 3.0 * whole, lanes
             assert _ms(lambda: p.solve_transpose(one)) < 3.0 * whole, lanes
         assert _ms(lambda: p.solve(b, algo=algo)) < 3.0 * _ms(lambda: p.solve(few, algo=algo))
+
+
+@pytest.mark.parametrize("lanes", [1, 2])
+def test_partitioned_solve_of_rows_that_differ(lanes):
+    """Parts of twenty rows, a row a group, up to a thousand entries of earlier parts: the
+    sliced copy would take two to three times as long as the level-ordered one."""
+    A = synth.general_lower(3001, 5)
+    b = torch.tensor(synth.uniform(A.n, 3), device=dev())
+    with plan_for(A) as p:
+        p.set_tuning(lanes, 256, 0)
+        assert torch.equal(p.solve(b, algo="partitioned"), p.solve(b, algo="self"))
+        assert (_ms(lambda: p.solve(b, algo="partitioned"))
+                < 1.5 * _ms(lambda: p.solve(b, algo="permuted")))
+
+
+def test_partitioned_solve_with_a_warp_per_short_row():
+    """32 lanes on rows of two entries: in place, not on the level-ordered copy, which
+    would take nearly twice as long."""
+    A = synth.lap2d_5pt_lower(1024, 1024)
+    b = torch.tensor(synth.uniform(A.n, 3), device=dev(), dtype=torch.float32)
+    with plan_for(A, dtype=torch.float32) as p:
+        p.set_tuning(32, 512, 0)
+        p.set_partition(4096, 4)
+        want = p.solve(b, algo="self")
+        assert torch.equal(p.solve(b, algo="partitioned"), want)
+        x = b.clone()
+        assert torch.equal(p.solve(x, out=x, algo="partitioned"), want)
+        assert (_ms(lambda: p.solve(b, algo="partitioned"))
+                < 1.4 * _ms(lambda: p.solve(b, algo="self")))
+        p.prepare("partitioned")
+        x = b.clone()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            p.solve(x, out=x, algo="partitioned")
+        g.replay()
+        assert torch.equal(x, want)
+
+
+def test_partitioned_solve_of_wide_levels_and_empty_slots():
+    A = synth.lap3d_7pt_lower(96, 96, 96)
+    b = torch.tensor(synth.uniform(A.n, 3), device=dev())
+    with plan_for(A) as p:
+        p.set_tuning(16, 512, 0)
+        p.set_partition(4096, 4)
+        assert torch.equal(p.solve(b, algo="partitioned"), p.solve(b, algo="self"))
+        assert (_ms(lambda: p.solve(b, algo="partitioned"))
+                < 1.4 * _ms(lambda: p.solve(b, algo="permuted")))
