@@ -54,6 +54,9 @@ struct Levels {
     int* pidx = nullptr;
     void* pvals = nullptr;
     void* xp = nullptr;
+    // (pkept, pstale: as with the sliced copies below; kept unless only partitioned
+    // solves have used it, slice_form)
+    bool pkept = false, pstale = false;
     // Column-wise solve (SPTRSV_ALGO_SELF_COLUMN, built on first use): the
     // dependency count of every row and the working counters.
     int* count0 = nullptr;
@@ -92,7 +95,13 @@ struct Levels {
         // FP32 values, for the FP32 solves of a refined F64 plan
         void* vals32 = nullptr;
         void* dinv32 = nullptr;
+        // Values change: the copy used last and the kept ones (prepared, or part of a
+        // captured graph, which reads it on every replay) are brought up to date at once,
+        // the others (stale) when they are used again.
+        bool kept = false, stale = false;
+        unsigned long long used = 0;  // qclock of the last use
     } qs[6];
+    unsigned long long qclock = 0;
     // FP32 values of the level-ordered copy and FP32 publication buffers of both
     // copies of an F64 plan, for the FP32 solves of the refined solve (built
     // on first use from the plan's FP32 copy of the values).
@@ -105,8 +114,11 @@ struct Levels {
     size_t xpm_bytes = 0;
 };
 
-// Sliced copies larger than this many times the stored entries are not built.
+// Sliced copies larger than this many times the stored entries are not built, and the
+// copies of several widths of one direction that nobody asked to keep are together no
+// larger: the ones used longest ago make room.
 constexpr long long kMaxPadding = 8;
+long long most_slots(long long nnz) { return kMaxPadding * nnz + (1 << 20); }
 constexpr int kSmallBlock = 512;  // threads of a solve in one block, and
 constexpr int kSmallGroups = 4;   // the row groups per level it is used for
 
@@ -689,12 +701,36 @@ int copy_diag(sptrsv_plan_t P, bool trans) {
     return (trans ? !P->upper : P->upper) ? 1 : 0;
 }
 
+// Values of the level-ordered copy from the plan's values, and of its FP32 version.
+cudaError_t refill_permuted(sptrsv_plan_t P, bool trans, cudaStream_t s) {
+    Levels& L = trans ? P->trn : P->fwd;
+    const int* ptr = trans ? P->tptr : P->rowptr;
+    const int* idx = trans ? P->tidx : P->colidx;
+    const int* vmap = trans ? P->tmap : nullptr;
+    const bool upper = trans ? !P->upper : P->upper;
+    cudaError_t e = launch_permute_rows(P->f64, P->n, ptr, idx, vmap, P->vals, L.jlev, L.ipos,
+                                        L.pptr, nullptr, L.pvals, P->num_sms * 16, s,
+                                        copy_diag(P, trans), upper);
+    if (e == cudaSuccess && L.pvals32 && P->vals32)
+        e = launch_permute_rows(false, P->n, ptr, idx, vmap, P->vals32, L.jlev, L.ipos, L.pptr,
+                                nullptr, L.pvals32, P->num_sms * 16, s, copy_diag(P, trans), upper);
+    if (e == cudaSuccess) L.pstale = false;
+    return e;
+}
+
 // Level-ordered copy of one direction's pattern and values (Sec. 4.3,
 // remark 2: preordering by level), its self-check and the publication
-// buffer.  Built once per direction; allocates and synchronises s.
-sptrsv_status_t build_permuted(sptrsv_plan_t P, bool trans, cudaStream_t s) {
+// buffer.  Built once per direction; allocates and synchronises s.  keep: its values are
+// brought up to date whenever the plan's change, not only before its next use.
+sptrsv_status_t build_permuted(sptrsv_plan_t P, bool trans, cudaStream_t s, bool keep = true) {
     Levels& L = trans ? P->trn : P->fwd;
-    if (L.pptr) return SPTRSV_OK;
+    L.pkept = L.pkept || keep;
+    if (L.pptr && !L.pstale) return SPTRSV_OK;
+    if (L.pptr) {
+        CK(refill_permuted(P, trans, s));
+        L.pstale = capturing(s);  // recorded, not run
+        return SPTRSV_OK;
+    }
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
     const int n = P->n, nnz = P->nnz;
     const size_t esize = P->f64 ? sizeof(double) : sizeof(float);
@@ -781,39 +817,38 @@ SliceParams slice_params(sptrsv_plan_t P, bool trans, const Levels::Slices& q) {
     return p;
 }
 
-// Re-gathers the values of every copy from the plan's values.
+// Values of a sliced copy from the plan's values.
+cudaError_t refill_slices(sptrsv_plan_t P, bool trans, int lanes, Levels::Slices& q,
+                          cudaStream_t s) {
+    cudaError_t e = launch_fill_slices(P->f64, slice_params(P, trans, q), lanes, q.grp, P->vals,
+                                       nullptr, q.vals, q.dinv, s);
+    if (e == cudaSuccess && q.vals32 && P->vals32)
+        e = launch_fill_slices(false, slice_params(P, trans, q), lanes, q.grp, P->vals32, nullptr,
+                               q.vals32, q.dinv32, s);
+    if (e == cudaSuccess) q.stale = false;
+    return e;
+}
+
+// Re-gathers the values of every copy from the plan's values, or marks those that are
+// neither kept nor the one that a partitioned solve used last for their next use.
 cudaError_t refresh_permuted(sptrsv_plan_t P, cudaStream_t s) {
     for (int d = 0; d < 2; ++d) {
         Levels& L = d ? P->trn : P->fwd;
-        if (!L.pvals) continue;
-        cudaError_t e = launch_permute_rows(P->f64, P->n, d ? P->tptr : P->rowptr,
-                                            d ? P->tidx : P->colidx, d ? P->tmap : nullptr,
-                                            P->vals, L.jlev, L.ipos, L.pptr, nullptr, L.pvals,
-                                            P->num_sms * 16, s, copy_diag(P, d),
-                                            d ? !P->upper : P->upper);
-        if (e != cudaSuccess) return e;
-    }
-    for (int d = 0; d < 2; ++d) {
-        Levels& L = d ? P->trn : P->fwd;
+        bool now = L.pkept;  // the level-ordered copy
         for (int w = 0; w < 6; ++w) {
             Levels::Slices& q = L.qs[w];
+            const bool last = q.built && q.used == L.qclock;
+            now = now || (last && q.form == Levels::kLevelOrder);
             if (!q.vals) continue;
-            cudaError_t e = launch_fill_slices(P->f64, slice_params(P, d, q), 1 << w, q.grp,
-                                               P->vals, nullptr, q.vals, q.dinv, s);
-            if (e == cudaSuccess && q.vals32 && P->vals32)
-                e = launch_fill_slices(false, slice_params(P, d, q), 1 << w, q.grp, P->vals32,
-                                       nullptr, q.vals32, q.dinv32, s);
+            q.stale = !q.kept && !last;
+            if (q.stale) continue;
+            const cudaError_t e = refill_slices(P, d, 1 << w, q, s);
             if (e != cudaSuccess) return e;
         }
-    }
-    // the level-ordered FP32 copies of the refined solve, from the refreshed FP32 values
-    for (int d = 0; d < 2 && P->vals32; ++d) {
-        Levels& L = d ? P->trn : P->fwd;
-        if (!L.pvals32) continue;
-        cudaError_t e = launch_permute_rows(
-            false, P->n, d ? P->tptr : P->rowptr, d ? P->tidx : P->colidx,
-            d ? P->tmap : nullptr, P->vals32, L.jlev, L.ipos, L.pptr, nullptr, L.pvals32,
-            P->num_sms * 16, s, copy_diag(P, d), d ? !P->upper : P->upper);
+        if (!L.pvals) continue;
+        L.pstale = !now;
+        if (L.pstale) continue;
+        const cudaError_t e = refill_permuted(P, d, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1111,11 +1146,27 @@ Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long s
     const double rows = (double)P->n * lanes / 32.0;  // groups if all were full
     if ((double)more[0] > (lengths_like(P, L) ? 16.0 : 1.25) * rows || (double)more[1] > 64.0 * rows)
         return Levels::kLevelOrder;
-    if (slots > kMaxPadding * P->nnz + (1 << 20))
+    if (slots > most_slots(P->nnz))
         return lanes == 32 ? Levels::kInPlace : Levels::kLevelOrder;
     if (4 * slots > 7ll * P->nnz && level_tickets(P, L, lanes) > 512.0)
         return Levels::kLevelOrder;
     return Levels::kSliced;
+}
+
+// Frees the copies of one direction used longest ago until those that are not kept and
+// `slots` more are at most `most`.  The caller has synchronised the stream of the solves.
+void make_room(Levels& L, long long slots, long long most) {
+    while (true) {
+        Levels::Slices* oldest = nullptr;
+        long long total = slots;
+        for (Levels::Slices& o : L.qs) {
+            if (!o.vals || o.kept) continue;
+            total += o.slots;
+            if (!oldest || o.used < oldest->used) oldest = &o;
+        }
+        if (total <= most || !oldest) return;
+        free_slices(*oldest);
+    }
 }
 
 // Sliced copy of one direction's matrix in part order (which must exist) for
@@ -1126,8 +1177,16 @@ Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long s
 sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_t s) {
     Levels& L = trans ? P->trn : P->fwd;
     const int w = log2_lanes(lanes);
-    if (L.qs[w].built) return SPTRSV_OK;
+    if (L.qs[w].built && !L.qs[w].stale) {
+        L.qs[w].used = ++L.qclock;
+        return SPTRSV_OK;
+    }
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
+    if (L.qs[w].built) {
+        CK(refill_slices(P, trans, lanes, L.qs[w], s));
+        L.qs[w].used = ++L.qclock;
+        return SPTRSV_OK;
+    }
     const int n = P->n;
     const size_t N = (size_t)n;
     const size_t esize = P->f64 ? sizeof(double) : sizeof(float);
@@ -1174,6 +1233,7 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
     if (e == cudaSuccess) q.form = slice_form(P, L, lanes, q.slots, h_more);
     const size_t slots = q.slots > 0 ? (size_t)q.slots : 1;
     if (e == cudaSuccess && q.form == Levels::kSliced) {
+        make_room(L, q.slots, most_slots(P->nnz));
         e = cudaMalloc(&q.cols, sizeof(int) * slots);
         if (e == cudaSuccess) e = cudaMalloc(&q.vals, esize * slots);
         if (e == cudaSuccess && !P->unit) e = cudaMalloc(&q.dinv, esize * N);
@@ -1208,6 +1268,7 @@ sptrsv_status_t build_slices(sptrsv_plan_t P, bool trans, int lanes, cudaStream_
         q.form = form;
     }
     q.built = true;
+    q.used = ++L.qclock;
     L.qs[w] = q;
     return SPTRSV_OK;
 }
@@ -1357,20 +1418,25 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     if (f64 != P->f64 && !f32_of_f64) return SPTRSV_ERR_INVALID_ARG;
     bool parts = algo == SPTRSV_ALGO_SELF_PARTITIONED && !mrhs;
     void* stand_in = nullptr;
+    bool keep_perm = true;
     if (parts) {
         ST(build_parts(P, trans, s));
-        // While s is being captured a copy cannot be built for another width than
-        // the one prepared: that solve runs in place (bitwise the same result).
-        const Levels& Lq = trans ? P->trn : P->fwd;
-        const Levels::Slices& q = Lq.qs[log2_lanes(lanes)];
+        // While s is being captured a copy cannot be built, nor brought up to date, for
+        // another width than the one prepared: that solve runs in place (bitwise the
+        // same result).
+        Levels& Lq = trans ? P->trn : P->fwd;
+        Levels::Slices& q = Lq.qs[log2_lanes(lanes)];
         bool in_place = false;
-        if (!f32_of_f64 && capturing(s) &&
-            (!q.built || (q.form == Levels::kLevelOrder && !Lq.pptr)))
+        const bool captured = capturing(s);
+        if (!f32_of_f64 && captured &&
+            (!q.built || q.stale || (q.form == Levels::kLevelOrder && (!Lq.pptr || Lq.pstale))))
             for (const Levels::Slices& o : Lq.qs) in_place = in_place || o.built;
         if (!in_place) {
             ST(build_slices(P, trans, lanes, s));
             in_place = q.form == Levels::kInPlace;
             parts = q.form == Levels::kSliced;
+            q.kept = q.kept || captured;  // the graph reads the copy on every replay
+            keep_perm = q.kept;
             if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
         }
         if (in_place) {
@@ -1383,7 +1449,7 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     // (a partitioned solve for which slice_form chose the level-ordered copy too)
     const bool permuted = (algo == SPTRSV_ALGO_SELF_PERMUTED || blocked ||
                            (algo == SPTRSV_ALGO_SELF_PARTITIONED && !parts)) && !mrhs;
-    if (permuted) ST(build_permuted(P, trans, s));
+    if (permuted) ST(build_permuted(P, trans, s, keep_perm));
     if (permuted && f32_of_f64) ST(build_copy_f32(P, trans, s));
     const bool column = algo == SPTRSV_ALGO_SELF_COLUMN && !mrhs;
     if (column) ST(build_column(P, trans, s));
@@ -1868,6 +1934,7 @@ sptrsv_status_t sptrsv_prepare(sptrsv_plan_t plan, int transpose, sptrsv_algo_t 
         case SPTRSV_ALGO_SELF_PARTITIONED:
             ST(build_parts(P, trans, s));
             ST(build_slices(P, trans, lanes, s));
+            (trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].kept = true;
             if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].form == Levels::kLevelOrder)
                 ST(build_permuted(P, trans, s));
             break;
