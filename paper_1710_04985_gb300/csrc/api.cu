@@ -820,11 +820,12 @@ SliceParams slice_params(sptrsv_plan_t P, bool trans, const Levels::Slices& q) {
 // Values of a sliced copy from the plan's values.
 cudaError_t refill_slices(sptrsv_plan_t P, bool trans, int lanes, Levels::Slices& q,
                           cudaStream_t s) {
-    cudaError_t e = launch_fill_slices(P->f64, slice_params(P, trans, q), lanes, q.grp, P->vals,
-                                       nullptr, q.vals, q.dinv, s);
+    const int longest = (trans ? P->trn : P->fwd).max_len - (P->unit ? 0 : 1);
+    cudaError_t e = launch_refill_slices(P->f64, slice_params(P, trans, q), lanes, longest, q.grp,
+                                         P->vals, q.cols, q.vals, q.dinv, s);
     if (e == cudaSuccess && q.vals32 && P->vals32)
-        e = launch_fill_slices(false, slice_params(P, trans, q), lanes, q.grp, P->vals32, nullptr,
-                               q.vals32, q.dinv32, s);
+        e = launch_refill_slices(false, slice_params(P, trans, q), lanes, longest, q.grp,
+                                 P->vals32, q.cols, q.vals32, q.dinv32, s);
     if (e == cudaSuccess) q.stale = false;
     return e;
 }

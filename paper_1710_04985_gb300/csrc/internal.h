@@ -237,6 +237,12 @@ cudaError_t launch_fill_slices(bool f64, const SliceParams& p, int lanes, const 
                                const void* vals, int* cols, void* out, void* dinv,
                                cudaStream_t s);
 
+// The values and 1/d(i) alone, into slices that launch_fill_slices wrote (cols).
+// longest: entries of the longest row beside the diagonal.
+cudaError_t launch_refill_slices(bool f64, const SliceParams& p, int lanes, int longest,
+                                 const int4* grp, const void* vals, const int* cols, void* out,
+                                 void* dinv, cudaStream_t s);
+
 // ---- level-ordered copy (permute.cu)
 // lens[k] = length of row jlev[k].
 cudaError_t launch_ordered_lengths(int n, const int* ptr, const int* jlev, int* lens,

@@ -260,7 +260,9 @@ __device__ __forceinline__ int part_of_group(const SliceParams& p, int g) {
 struct FoldRow {
     int i, q0, m, len;
 };
-__device__ __forceinline__ FoldRow fold_row(const SliceParams& p, int k, bool has) {
+// (stored: a diagonal is known to be)
+__device__ __forceinline__ FoldRow fold_row(const SliceParams& p, int k, bool has,
+                                            bool stored = false) {
     FoldRow r = {-1, 0, 0, 0};
     if (!has) return r;
     r.i = p.qord[k];
@@ -268,7 +270,7 @@ __device__ __forceinline__ FoldRow fold_row(const SliceParams& p, int k, bool ha
     r.len = end - beg;
     r.q0 = p.upper ? end - 1 : beg;
     r.m = r.len;
-    if (r.len > 0 && p.idx[p.upper ? beg : end - 1] == r.i) --r.m;
+    if (r.len > 0 && (stored || p.idx[p.upper ? beg : end - 1] == r.i)) --r.m;
     return r;
 }
 
@@ -369,6 +371,82 @@ __global__ void fill_slices_k(SliceParams p, const int4* __restrict__ grp,
             out[at] = a;
         }
         if (t < r.m) report(p.status, r.i, kCodeInternal);  // an entry found no slice
+    }
+}
+
+// The values alone, into slices that are there: the columns say which slots hold an
+// entry, so that a batch of a lane's entries is loaded at once and the next batch's
+// columns meanwhile (fill_slices_k looks at one entry after the other to tell which
+// slice it belongs to, a load's latency per slice of a long row).  Values of one copy,
+// both kernels, us: general 3001 rows FP64, 4 and 8 lanes 141 -> 69 and 94 -> 41, of
+// 100001 rows 195 -> 97 and 134 -> 65; band of 40, 4 lanes 49 -> 34.  Where rows take a few
+// slices of a large system, the columns are traffic on top (5-point 1024 x 1024 FP32, one
+// lane 101 and 141; 7-point 96^3, 4 lanes 74 and 101): those keep fill_slices_k.
+template <typename T, int W>
+__global__ void refill_slices_k(SliceParams p, const int4* __restrict__ grp,
+                                const T* __restrict__ vals, const int* __restrict__ cols, T* out,
+                                T* dinv) {
+    constexpr int U = 8;
+    const int lane = threadIdx.x & 31, grow = lane / W, sl = lane % W;
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < p.ngroups;
+         g += warps) {
+        const int4 d = grp[g];
+        const int cnt = d.w & 63, X = d.z, S = d.z + (d.w >> 12), k = d.x + grow;
+        const FoldRow r = fold_row(p, k, grow < cnt, dinv != nullptr);
+        T di = T(1);
+        if (dinv && r.len > 0) {
+            const int qd = p.upper ? r.q0 - r.m : r.q0 + r.m;  // the diagonal folds last
+            di = T(1) / vals[p.vmap ? p.vmap[qd] : qd];
+            if (sl == 0) dinv[k] = di;
+        }
+        int t = sl, c[U], cn[U];
+        const long long at = (long long)d.y * 32 + lane;
+        auto load_cols = [&](int s) {  // the warp's slices s, s + 1, ...
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s + u >= S) break;
+                cn[u] = cols[at + 32ll * (s + u)];
+            }
+        };
+        load_cols(0);
+        for (int s = 0; s < S; s += U) {
+            int q[U];
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s + u >= S) break;
+                c[u] = cn[u];
+            }
+            load_cols(s + U);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s + u >= S) break;
+                q[u] = -1;
+                if (c[u] != (s + u < X ? -1 : p.max_part)) {
+                    q[u] = p.upper ? r.q0 - t : r.q0 + t;
+                    t += W;
+                }
+            }
+            if (p.vmap) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (s + u >= S) break;
+                    if (q[u] >= 0) q[u] = p.vmap[q[u]];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s + u >= S) break;
+                v[u] = q[u] >= 0 ? vals[q[u]] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s + u >= S) break;  // an FP64 multiply takes 64 cycles, needed or not
+                const T a = dinv ? v[u] * di : v[u];
+                if (q[u] >= 0) out[at + 32ll * (s + u)] = a;
+            }
+        }
     }
 }
 
@@ -525,6 +603,34 @@ cudaError_t launch_fill_slices(bool f64, const SliceParams& p, int lanes, const 
                                cudaStream_t s) {
     return f64 ? fill_t<double>(p, lanes, grp, vals, cols, out, dinv, s)
                : fill_t<float>(p, lanes, grp, vals, cols, out, dinv, s);
+}
+
+template <typename T>
+static cudaError_t refill_t(const SliceParams& p, int lanes, const int4* grp, const void* vals,
+                            const int* cols, void* out, void* dinv, cudaStream_t s) {
+    const int g = warps_grid(p.ngroups);
+#define SPTRSV_REFILL(W) \
+    refill_slices_k<T, W><<<g, 256, 0, s>>>(p, grp, (const T*)vals, cols, (T*)out, (T*)dinv)
+    switch (lanes) {
+        case 1: SPTRSV_REFILL(1); break;
+        case 2: SPTRSV_REFILL(2); break;
+        case 4: SPTRSV_REFILL(4); break;
+        case 8: SPTRSV_REFILL(8); break;
+        case 16: SPTRSV_REFILL(16); break;
+        case 32: SPTRSV_REFILL(32); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef SPTRSV_REFILL
+    return cudaGetLastError();
+}
+
+cudaError_t launch_refill_slices(bool f64, const SliceParams& p, int lanes, int longest,
+                                 const int4* grp, const void* vals, const int* cols, void* out,
+                                 void* dinv, cudaStream_t s) {
+    if (lanes <= 8 && longest <= 4 * lanes && p.n > 300000)
+        return launch_fill_slices(f64, p, lanes, grp, vals, nullptr, out, dinv, s);
+    return f64 ? refill_t<double>(p, lanes, grp, vals, cols, out, dinv, s)
+               : refill_t<float>(p, lanes, grp, vals, cols, out, dinv, s);
 }
 
 #undef SPTRSV_LAUNCH

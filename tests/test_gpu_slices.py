@@ -112,3 +112,16 @@ def test_copies_of_several_widths_are_bounded():
         assert free - torch.cuda.mem_get_info()[0] <= 12 * (8 * A.nnz + 2**20) + beside
         p.set_tuning(1, 256, 0)
         assert torch.equal(p.solve(b, algo="partitioned"), want)
+
+
+def test_an_update_of_long_rows():
+    """About as long as that of the level-ordered copy (three times as long, one entry
+    after the other)."""
+    A = synth.general_lower(3001, 5)
+    b = torch.tensor(synth.uniform(A.n, 67), device=dev())
+    with plan_for(A) as p, plan_for(A) as q:
+        p.set_tuning(16, 256, 0)
+        p.set_partition(4096, 1)
+        p.solve(b, algo="partitioned")
+        q.solve(b, algo="permuted")
+        assert _ms(lambda: p.set_values(p.vals)) < 2.0 * _ms(lambda: q.set_values(q.vals))
