@@ -95,6 +95,7 @@ struct Levels {
         // FP32 values, for the FP32 solves of a refined F64 plan
         void* vals32 = nullptr;
         void* dinv32 = nullptr;
+        bool no_room32 = false;
         // Values change: the copy used last and the kept ones (prepared, or part of a
         // captured graph, which reads it on every replay) are brought up to date at once,
         // the others (stale) when they are used again.
@@ -1301,16 +1302,19 @@ sptrsv_status_t build_copy_f32(sptrsv_plan_t P, bool trans, cudaStream_t s) {
     return SPTRSV_OK;
 }
 
-// The same for the sliced copy of one width.
+// The same for the sliced copy of one width.  Its slots may be several times the stored
+// entries: where there is no room for them, SPTRSV_ERR_OOM at once from then on.
 sptrsv_status_t build_slices_f32(sptrsv_plan_t P, bool trans, int lanes, cudaStream_t s) {
     Levels& L = trans ? P->trn : P->fwd;
     Levels::Slices& q = L.qs[log2_lanes(lanes)];
     if (q.vals32 && L.xq32) return SPTRSV_OK;
+    if (q.no_room32) return SPTRSV_ERR_OOM;
     if (!P->vals32 && P->nnz > 0) return SPTRSV_ERR_NOT_SUPPORTED;
     if (capturing(s)) return SPTRSV_ERR_NOT_SUPPORTED;
-    if (!L.xq32) CK(cudaMalloc(&L.xq32, sizeof(float) * (size_t)P->n));
     void *v = nullptr, *di = nullptr;
-    cudaError_t e = cudaMalloc(&v, sizeof(float) * (q.slots > 0 ? (size_t)q.slots : 1));
+    cudaError_t e = cudaSuccess;
+    if (!L.xq32) e = cudaMalloc(&L.xq32, sizeof(float) * (size_t)P->n);
+    if (e == cudaSuccess) e = cudaMalloc(&v, sizeof(float) * (q.slots > 0 ? (size_t)q.slots : 1));
     if (e == cudaSuccess && !P->unit) e = cudaMalloc(&di, sizeof(float) * (size_t)P->n);
     if (e == cudaSuccess)
         e = launch_fill_slices(false, slice_params(P, trans, q), lanes, q.grp, P->vals32, nullptr,
@@ -1318,6 +1322,8 @@ sptrsv_status_t build_slices_f32(sptrsv_plan_t P, bool trans, int lanes, cudaStr
     if (e != cudaSuccess) {
         cudaFree(v);
         cudaFree(di);
+        q.no_room32 = e == cudaErrorMemoryAllocation;
+        if (q.no_room32) cudaGetLastError();  // this call's own: the solve goes on in place
         return cuda_fail(e);
     }
     q.vals32 = v;
@@ -1438,7 +1444,11 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
             parts = q.form == Levels::kSliced;
             q.kept = q.kept || captured;  // the graph reads the copy on every replay
             keep_perm = q.kept;
-            if (parts && f32_of_f64) ST(build_slices_f32(P, trans, lanes, s));
+            if (parts && f32_of_f64) {
+                const sptrsv_status_t rc = build_slices_f32(P, trans, lanes, s);
+                in_place = rc == SPTRSV_ERR_OOM;  // in place takes nothing more
+                if (!in_place) ST(rc);
+            }
         }
         if (in_place) {
             stand_in = Lq.xq;  // the publication buffer of the parts holds b

@@ -1,5 +1,5 @@
 """What the library asks of the CUDA runtime, seen and steered by a shim in front
-of libcudart: limits of a kernel that all plans of a process share, and queries
+of libcudart: limits of a kernel that all plans of a process share, and calls
 that fail.  The shim is preloaded into a child process, once for all tests."""
 import json
 import os
@@ -51,6 +51,14 @@ cudaError_t cudaGetLastError(void) {
     return real();
 }
 
+/* allocations of this many bytes and more fail (0: none) */
+static size_t fail_from;
+void shim_fail_malloc_from(size_t bytes) { fail_from = bytes; }
+cudaError_t cudaMalloc(void** p, size_t bytes) {
+    REAL(cudaMalloc);
+    return fail_from && bytes >= fail_from ? cudaErrorMemoryAllocation : real(p, bytes);
+}
+
 /* clusters: a size whose query fails, and the last one launched */
 static unsigned refused, launched;
 void shim_refuse_cluster(unsigned blocks) { refused = blocks; }
@@ -80,6 +88,7 @@ import synth
 from gpu_util import dev, plan_for
 
 shim = ctypes.CDLL(sys.argv[2])
+shim.shim_fail_malloc_from.argtypes = [ctypes.c_size_t]
 out = {}
 
 
@@ -124,7 +133,25 @@ def cluster():
     shim.shim_refuse_cluster(0)
 
 
-for f in (one_block, cluster):
+def no_room():
+    A = synth.lap3d_7pt_ilu0(40, 41, 43)[0]
+    b = rhs(A)
+    with plan_for(A) as p, plan_for(A) as q:
+        for plan in (p, q):
+            plan.set_tuning(8, 256, 0)              # twice as many slots as entries
+            plan.best_algo = "partitioned"
+        want, _, _ = p.solve_refined(b)
+        q.solve(b, algo="partitioned")              # its FP64 copy is there
+        shim.shim_fail_malloc_from(6 * A.nnz)       # room for nnz floats, not for the slices
+        try:
+            got, _, _ = q.solve_refined(b)
+            out["refined"] = bool(torch.equal(got, want))
+        except Exception as e:
+            out["refined"] = repr(e)
+        shim.shim_fail_malloc_from(0)
+
+
+for f in (one_block, cluster, no_room):
     f()
 print(json.dumps(out))
 """
@@ -161,6 +188,10 @@ def test_a_cluster_size_that_cannot_be_asked_for_leaves_the_smaller_one(seen):
 def test_asking_for_the_cluster_size_clears_no_error_of_the_caller(seen):
     first, later = seen["last_errors"]
     assert first == later
+
+
+def test_refined_solve_without_room_for_the_fp32_slices(seen):
+    assert seen["refined"] is True
 
 
 def test_two_threads_with_plans_of_their_own(cuda_device):
