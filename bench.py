@@ -77,7 +77,7 @@ def kernel_source_sha(algo="self"):
     """Hash of the code (not the comments) of a solve kernel's source file and
     the shared headers: an ncu figure taken on other code is not reused."""
     h = hashlib.sha256()
-    for f in (KERNELS[algo][1], "common.cuh", "internal.h", "self_rows.cuh"):
+    for f in (KERNELS[algo][1], "common.cuh", "internal.h", "self_rows.cuh", "cursor.h"):
         with open(os.path.join(ROOT, "paper_1710_04985_gb300", "csrc", f)) as fh:
             h.update(_code_only(fh.read()).encode())
     return h.hexdigest()[:12]

@@ -145,27 +145,35 @@ typedef enum {
                                      levels.  Bitwise equal to SPTRSV_ALGO_SELF for
                                      equal lanes.  More right-hand sides run as with
                                      SPTRSV_ALGO_SELF_PERMUTED                           */,
-    SPTRSV_ALGO_SELF_PARTITIONED = 7  /* the blocked solve of SPTRSV_ALGO_SELF_BLOCKED
-                                     on a part-ordered copy: the substitution order is
-                                     split where the matrix decouples (every system
-                                     boundary of a block-diagonal batch), long blocks
-                                     are cut into parts of at most part_rows
-                                     consecutive rows (sptrsv_set_partition), short
-                                     ones packed together; parts are listed in the
+    SPTRSV_ALGO_SELF_PARTITIONED = 7  /* Alg. 3 on a part-ordered copy in slices: the
+                                     substitution order is split where the matrix
+                                     decouples (every system boundary of a block-diagonal
+                                     batch), long blocks are cut into parts of at most
+                                     part_rows consecutive rows (sptrsv_set_partition),
+                                     short ones packed together; parts are listed in the
                                      order they are handed out (see
                                      sptrsv_partition_info) and by level (Sec. 4.1)
-                                     inside a part, and a thread block takes one part
-                                     per tile, so a dependency inside the part passes
-                                     through shared memory and only dependencies on
-                                     earlier parts wait on published values in L2
-                                     (Alg. 3).  On a grid in natural order a part is a
-                                     slab of grid lines.  Built on first use (a copy of
-                                     the pattern and values, same value snapshot as
-                                     SPTRSV_ALGO_SELF_PERMUTED, allocates and
-                                     synchronises; not during graph capture) and again
-                                     when the part size changes.  Bitwise equal to
-                                     SPTRSV_ALGO_SELF for equal lanes.  More right-hand
-                                     sides run as with SPTRSV_ALGO_SELF_PERMUTED         */,
+                                     inside a part, and a thread block of at most 512
+                                     threads (larger block sizes run as 512) takes one
+                                     part, so a dependency inside the part passes through
+                                     shared memory and only dependencies on earlier parts
+                                     wait on published values in L2 (Alg. 3).  On a grid
+                                     in natural order a part is a slab of grid lines.
+                                     Built on first use of a width (lanes_per_row; same
+                                     value snapshot as SPTRSV_ALGO_SELF_PERMUTED,
+                                     allocates and synchronises; a solve captured at a
+                                     width that is not there runs in place) and again
+                                     when the part size changes.  Memory: up to 8 slots
+                                     (a value and a column each) per stored entry and
+                                     direction for all widths that were not prepared
+                                     (sptrsv_prepare) or captured, the ones used longest
+                                     ago making room; a prepared or captured width is
+                                     kept.  Where its slots would be mostly empty or long
+                                     rows would be taken one after another, a width runs
+                                     on the level-ordered copy or in place instead.
+                                     Bitwise equal to SPTRSV_ALGO_SELF for equal lanes.
+                                     More right-hand sides run as with
+                                     SPTRSV_ALGO_SELF_PERMUTED                           */,
     SPTRSV_ALGO_AUTO = 8          /* the plan's default form (sptrsv_set_default_algo;
                                      SPTRSV_ALGO_SELF until one is set), e.g. the one an
                                      autotuner measured fastest                          */
@@ -208,8 +216,8 @@ typedef enum {
 /* ------------------------------------------------------------------ setup */
 
 /* Largest matrix order and number of stored entries: 2^31 - 256.  A solve
- * kernel's cursor over a row's entries may run up to 128 entries past the
- * row's end and stays a 32-bit int. */
+ * kernel's index of a row's entries may run up to 255 entries past the row's
+ * end and stays a 32-bit int. */
 #define SPTRSV_MAX_SIZE 2147483392
 
 /* Setup phase (Sec. 4.4, Table 1): validates the CSR (Sec. 3), builds the
@@ -378,8 +386,9 @@ SPTRSV_API sptrsv_status_t sptrsv_set_values(sptrsv_plan_t plan, const void *d_v
 /* Re-reads d_vals into every copy of the values the plan holds: the FP32
  * copy of sptrsv_solve_refined, the level-ordered copy of
  * SPTRSV_ALGO_SELF_PERMUTED / _BLOCKED (and of their multi-RHS solves), the
- * part-ordered copy of SPTRSV_ALGO_SELF_PARTITIONED, and the FP32 versions of
- * both copies that refined solves use.  Solves of those forms read the copies,
+ * part-ordered copies of SPTRSV_ALGO_SELF_PARTITIONED (those of widths that
+ * were neither prepared nor captured nor used last follow at their next
+ * solve), and the FP32 versions of the copies that refined solves use.  Solves of those forms read the copies,
  * not d_vals: after changing d_vals in place, call this (on the solves'
  * stream, or synchronise) before the next solve.  Async. */
 SPTRSV_API sptrsv_status_t sptrsv_refresh_values(sptrsv_plan_t plan, void *stream);

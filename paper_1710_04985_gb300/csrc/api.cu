@@ -1140,8 +1140,10 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
 //  * more than seven in eight slots would be empty (kMaxPadding): with 32 lanes in place
 //    (5-point 1024 x 1024, FP64: 1.72 ms, level-ordered 2.35, the kernel before 1.87),
 //    else level-ordered (band of 40, one lane: 28.1 ms, in place 32.5);
-//  * levels are wide (more than 512 tickets), so that the empty slots count, and nearly
-//    half of them are empty (7-point 96^3, 16 lanes: 0.97 ms, level-ordered 0.54).
+//  * rows are alike and levels wide (more than 512 tickets), so that the empty slots count,
+//    and nearly half of them are empty (7-point 96^3, 16 lanes: 0.97 ms, level-ordered
+//    0.54; but 512 general systems with 8 lanes, whose levels are wide because they are
+//    many: 3.2 ms, level-ordered 7 and more).
 // All three give bitwise the same result.
 Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long slots,
                         const unsigned long long* more) {
@@ -1150,7 +1152,7 @@ Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long s
         return Levels::kLevelOrder;
     if (slots > most_slots(P->nnz))
         return lanes == 32 ? Levels::kInPlace : Levels::kLevelOrder;
-    if (4 * slots > 7ll * P->nnz && level_tickets(P, L, lanes) > 512.0)
+    if (lengths_like(P, L) && 4 * slots > 7ll * P->nnz && level_tickets(P, L, lanes) > 512.0)
         return Levels::kLevelOrder;
     return Levels::kSliced;
 }

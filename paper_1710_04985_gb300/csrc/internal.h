@@ -131,7 +131,7 @@ cudaError_t launch_blocked_k1(bool f64, int lanes, const SolveParams& p, int til
                               int block, cudaStream_t s);
 // Blocks of one launch that can be resident at once (0: the shape cannot run).
 int blocked_resident_blocks(bool f64, int lanes, int block, int tile_rows, int num_sms);
-// Partitioned solve on the sliced copy (solve_partitioned.cu): a block per part
+// Partitioned solve on the sliced copy (solve_partitioned.cuh): a block per part
 // of at most p.max_part positions (p.max_part * element size at most the
 // device's opt-in shared memory per block, minus 128 B).  cluster in
 // {1, 2, 4, 8}: clusters of that many blocks take consecutive parts together

@@ -29,7 +29,7 @@
 // fold (no lane reduction to wait for).  The dependencies of a row on earlier
 // tiles are spread over its entries here (a level-ordered row names positions
 // of any earlier tile between positions of its own), unlike on the
-// part-ordered copy, whose kernel (solve_partitioned.cu) waits for them first.
+// part-ordered copy, whose kernel (solve_partitioned.cuh) waits for them first.
 #include "internal.h"
 
 namespace sptrsv {

@@ -8,7 +8,7 @@
 // level (Sec. 4.1), then row; every column index is renumbered to its
 // position in that order, or in its part (the sliced copy, below).  A dependency then points to an earlier position,
 // one inside the part to a row of a lower level of the same part.  The
-// partitioned kernel (solve_partitioned.cu) runs on this copy, one part per
+// partitioned kernel (solve_partitioned.cuh) runs on this copy, one part per
 // thread block: the block holds its part's unknowns in shared memory,
 // where dependencies inside the part are served, and waits for earlier parts
 // through the published values as in Alg. 3.  On a structured grid in natural

@@ -103,3 +103,15 @@ def test_partitioned_solve_of_wide_levels_and_empty_slots():
         assert torch.equal(p.solve(b, algo="partitioned"), p.solve(b, algo="self"))
         assert (_ms(lambda: p.solve(b, algo="partitioned"))
                 < 1.4 * _ms(lambda: p.solve(b, algo="permuted")))
+
+
+def test_partitioned_solve_of_many_general_systems():
+    """Wide levels because the systems are many: the slices take less than half of what the
+    level-ordered copy takes."""
+    A = synth.block_diagonal([synth.general_lower(4000, 5)] * 200)
+    b = torch.tensor(synth.uniform(A.n, 3), device=dev())
+    with plan_for(A) as p:
+        p.set_tuning(8, 512, 0)
+        assert torch.equal(p.solve(b, algo="partitioned"), p.solve(b, algo="self"))
+        assert (_ms(lambda: p.solve(b, algo="partitioned"))
+                < 0.8 * _ms(lambda: p.solve(b, algo="permuted")))
