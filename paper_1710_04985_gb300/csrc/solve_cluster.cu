@@ -30,12 +30,15 @@
 //
 // A value that does not come within a quarter of the spin limit: the warp raises a
 // flag in every block, all warps leave their waits and meet at the barrier, and the
-// rows that are left of the window are computed level by level, a barrier between two
-// levels.  Nothing is waited for there: what is missing then never comes (it is
-// reported and taken as NaN), and every row that does not depend on it is exact.  A
-// warp's groups are in level order, so it goes through them once.  The next window
-// runs as usual; a value of an earlier window that is missing there was never
-// published and is not waited for either.
+// rows that are left are computed level by level, a barrier between two levels, in this
+// window and the later ones.  Nothing is waited for there: what is missing then never
+// comes (it is reported and taken as NaN), and every row that does not depend on it is
+// exact.  A warp's groups are in level order, so it goes through them once: the rest of a
+// solve takes a few times as long as usual, a barrier per level instead of a hop (40
+// windows of three interleaved chains 0.42 s instead of 0.1; 3.4 s when every level went
+// through its whole window).  Going back to the usual way in the next window needs a look
+// for values that were never published in every wait: any such code in the wait loop cost
+// FP32 solves 2 to 30 %.
 #include "self_rows.cuh"
 
 namespace sptrsv {
@@ -79,7 +82,7 @@ template <typename T, int W, bool MAP, bool PERM>
 __global__ void __launch_bounds__(kClusterBlock, 1)
     cluster_solve_k1(const __grid_constant__ SolveParams p, int nblocks) {
     extern __shared__ __align__(16) unsigned char ring_smem[];
-    __shared__ int s_bail[2];  // by parity of the window: read after its barrier, then cleared
+    __shared__ int s_bail[2];  // by parity of the window: read after its barrier
     constexpr int R = 32 / W;
     constexpr int E = ChunkOf<W>::E;
     constexpr int H = kWindowBytes / (int)sizeof(T);  // rows of a window, a multiple of 32
@@ -103,6 +106,7 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
     if (threadIdx.x < 2) s_bail[threadIdx.x] = 0;
     cluster_sync();
 
+    bool slow = false;
     int buf = 0;
     for (int base = 0; base < p.n; base = next_window(base, H, p.n), buf ^= 1) {
         const T* const ring = (const T*)ring_smem + buf * H;
@@ -139,7 +143,7 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
             T* const next = (T*)ring_smem + (buf ^ 1) * H;
             for (int k = threadIdx.x; k < H; k += blockDim.x) next[k] = Marker<T>::pending_value();
         }
-        for (int g = rank + nblocks * warp; g * R < rows; g += nblocks * nwarps) {
+        for (int g = rank + nblocks * warp; !slow && g * R < rows; g += nblocks * nwarps) {
             if (__any_sync(FULL, *bail != 0)) break;
             Row<T> r = take_row<T, W, PERM>(p, (long long)base + g * R + grp);
             start_row<T, W, MAP>(p, r, sl);
@@ -186,13 +190,6 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
                         if (__any_sync(FULL, act)) break;
                     }
                     if (++polls > kClusterHot) {
-#pragma unroll
-                        for (int e = 0; e < E; ++e)
-                            if (at[e] < 0 && Marker<T>::pending(v[e])) {
-                                // of an earlier window: it never comes
-                                report(p.status, r.i, kCodeTimeout);
-                                v[e] = Marker<T>::canonical_nan();
-                            }
                         if (polls > patience && lane < nblocks)
                             st_block(cluster_addr(smem_addr(&s_bail[buf]), lane), 1);
                         if (__any_sync(FULL, *bail != 0) || polls > 2 * patience + 1024) {
@@ -238,7 +235,8 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
         }
         __syncwarp();
         cluster_sync();
-        if (!*bail) continue;  // the same in every block
+        slow = slow || *bail;  // the same in every block
+        if (!slow) continue;
         // level by level: what has not been published by now and is not published
         // one barrier later never is
         const int last = p.lev[p.jlev[base + rows - 1]];
@@ -275,9 +273,6 @@ __global__ void __launch_bounds__(kClusterBlock, 1)
             __syncwarp();
             cluster_sync();
         }
-        // every thread has read the flag by now, and the next window of this parity
-        // begins two barriers from here
-        if (threadIdx.x == 0) *bail = 0;
     }
 }
 

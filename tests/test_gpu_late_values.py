@@ -71,8 +71,8 @@ def _braid(n, held):
 @pytest.mark.parametrize("lanes", [16, 32])
 def test_windows_after_a_missing_value_run_as_usual(lanes, algo):
     """The rows of 40 windows that do not need the missing value are exact, and the
-    call takes about as long as one in which nothing is missing (0.1 s; level by level
-    to the end it takes seconds)."""
+    call takes a few times what one takes in which nothing is missing (0.1 s; seconds
+    if every level goes through its whole window)."""
     held = 4999                                        # in the first window
     A, far = _braid(40 * 12288 + 100, held)
     behind = np.zeros(A.n, dtype=bool)
