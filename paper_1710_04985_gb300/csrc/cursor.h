@@ -13,20 +13,22 @@ namespace sptrsv {
 
 // A lane's cursor over the entries [.., end) of its row, `step` further on.  The lanes
 // of a warp go through chunks together, for as long as its longest row lasts: the
-// cursor of a lane whose row has ended stays where it is, less than a step past the
-// end, instead of running on by the length of its neighbour's row.
+// cursor of a lane whose row has ended stops 32 past the end instead of running on by the
+// length of its neighbour's row.  (Stepping only lanes that are inside their row is the
+// same, but cost the 27-point adjoint with one lane per row 10 %.)
 SPTRSV_HD int advance(int cursor, int step, int end) {
-    return cursor < end ? cursor + step : cursor;
+    const int next = cursor + step, most = end + 32;
+    return next < most ? next : most;
 }
 
 // An entry index that a kernel forms is at most this far past the end of its row (the
 // kernels assert it for their chunks): it stays an int at the limit.
 constexpr int kCursorAhead = 255;
 
-// The furthest for chunks of `slots` slots of `lanes` entries: a cursor that has just
-// been advanced past the end, the chunk after its own, the last slot of it.
+// The furthest for chunks of `slots` slots of `lanes` entries: a cursor that has stopped,
+// the chunk after its own, the last slot of it.
 constexpr int cursor_ahead(int lanes, int slots) {
-    return (lanes * slots - 1) + lanes * slots + lanes * (slots - 1);
+    return 32 + lanes * slots + lanes * (slots - 1);
 }
 
 // The start of the window of `rows` rows after the one at `base`, or n after the last
