@@ -834,24 +834,32 @@ cudaError_t refill_slices(sptrsv_plan_t P, bool trans, int lanes, Levels::Slices
 // Re-gathers the values of every copy from the plan's values, or marks those that are
 // neither kept nor the one that a partitioned solve used last for their next use.
 cudaError_t refresh_permuted(sptrsv_plan_t P, cudaStream_t s) {
+    // A recorded update runs on every replay, when nothing is marked: it covers every copy
+    // there is, and the graph holds their addresses.  It has not run yet.
+    const bool recorded = capturing(s);
     for (int d = 0; d < 2; ++d) {
         Levels& L = d ? P->trn : P->fwd;
         bool now = L.pkept;  // the level-ordered copy
         for (int w = 0; w < 6; ++w) {
             Levels::Slices& q = L.qs[w];
-            const bool last = q.built && q.used == L.qclock;
+            const bool last = q.built && q.used == L.qclock, before = q.stale;
             now = now || (last && q.form == Levels::kLevelOrder);
             if (!q.vals) continue;
+            q.kept = q.kept || recorded;
             q.stale = !q.kept && !last;
             if (q.stale) continue;
             const cudaError_t e = refill_slices(P, d, 1 << w, q, s);
             if (e != cudaSuccess) return e;
+            if (recorded) q.stale = before;
         }
         if (!L.pvals) continue;
-        L.pstale = !now;
+        const bool before = L.pstale;
+        L.pkept = L.pkept || recorded;
+        L.pstale = !now && !recorded;
         if (L.pstale) continue;
         const cudaError_t e = refill_permuted(P, d, s);
         if (e != cudaSuccess) return e;
+        if (recorded) L.pstale = before;
     }
     return cudaSuccess;
 }

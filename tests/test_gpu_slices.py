@@ -125,3 +125,33 @@ def test_an_update_of_long_rows():
         p.solve(b, algo="partitioned")
         q.solve(b, algo="permuted")
         assert _ms(lambda: p.set_values(p.vals)) < 2.0 * _ms(lambda: q.set_values(q.vals))
+
+
+def test_a_recorded_update_covers_every_copy_on_every_replay():
+    """New values and a solve at one width in a graph; solves at another width, and on the
+    level-ordered copy, see the values of each replay, also once their copies had to make
+    room for others'."""
+    A = synth.lap3d_7pt_ilu0(21, 23, 19)[0]
+    b = torch.tensor(synth.uniform(A.n, 69), device=dev())
+    with plan_for(A) as p:
+        for lanes in (2, 4):
+            p.set_tuning(lanes, 256, 0)
+            p.solve(b, algo="partitioned")
+        p.solve(b, algo="permuted")
+        x = torch.empty_like(b)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            p.vals.mul_(2.0)
+            p.refresh_values()
+            p.solve(b, out=x, algo="partitioned")
+        for lanes in (1, 8, 16):             # other copies, after the capture
+            p.set_tuning(lanes, 256, 0)
+            p.solve(b, algo="partitioned")
+        for _ in range(3):
+            g.replay()
+            for lanes in (2, 4):
+                p.set_tuning(lanes, 256, 0)
+                want = p.solve(b, algo="self")
+                assert torch.equal(p.solve(b, algo="partitioned"), want), lanes
+                assert torch.equal(p.solve(b, algo="permuted"), want), lanes
+            assert torch.equal(x, want)
