@@ -162,8 +162,10 @@ typedef enum {
                                      Built on first use of a width (lanes_per_row; same
                                      value snapshot as SPTRSV_ALGO_SELF_PERMUTED,
                                      allocates and synchronises; a solve captured at a
-                                     width that is not there runs in place) and again
-                                     when the part size changes.  Memory: up to 8 slots
+                                     width that is not there runs on the level-ordered
+                                     copy or, without one, in place, reading the array
+                                     of values of the capture) and again when the part
+                                     size changes.  Memory: up to 8 slots
                                      (a value and a column each) per stored entry and
                                      direction for all widths that were not prepared
                                      (sptrsv_prepare) or captured, the ones used longest

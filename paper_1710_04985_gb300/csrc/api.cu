@@ -1439,20 +1439,23 @@ sptrsv_status_t run_solve(sptrsv_plan_t P, bool trans, bool f64, const void* val
     if (parts) {
         ST(build_parts(P, trans, s));
         // While s is being captured a copy cannot be built, nor brought up to date, for
-        // another width than the one prepared: that solve runs in place (bitwise the
-        // same result).
+        // another width than the one prepared: that solve runs on the level-ordered copy
+        // or, where that is not there either, in place (bitwise the same result).  A width
+        // that runs in place otherwise takes the copy too: a captured solve in place goes
+        // on reading the array of values of its capture when the plan is given another.
         Levels& Lq = trans ? P->trn : P->fwd;
         Levels::Slices& q = Lq.qs[log2_lanes(lanes)];
-        bool in_place = false;
-        const bool captured = capturing(s);
-        if (!f32_of_f64 && captured &&
-            (!q.built || q.stale || (q.form == Levels::kLevelOrder && (!Lq.pptr || Lq.pstale))))
-            for (const Levels::Slices& o : Lq.qs) in_place = in_place || o.built;
-        if (!in_place) {
+        bool in_place = false, any = false;
+        for (const Levels::Slices& o : Lq.qs) any = any || o.built;
+        if (capturing(s) && !f32_of_f64 && any &&
+            (!q.built || q.stale || q.form != Levels::kSliced)) {
+            parts = false;
+            in_place = !Lq.pptr || Lq.pstale;
+        } else {
             ST(build_slices(P, trans, lanes, s));
             in_place = q.form == Levels::kInPlace;
             parts = q.form == Levels::kSliced;
-            q.kept = q.kept || captured;  // the graph reads the copy on every replay
+            q.kept = q.kept || capturing(s);  // the graph reads the copy on every replay
             keep_perm = q.kept;
             if (parts && f32_of_f64) {
                 const sptrsv_status_t rc = build_slices_f32(P, trans, lanes, s);
@@ -1956,7 +1959,7 @@ sptrsv_status_t sptrsv_prepare(sptrsv_plan_t plan, int transpose, sptrsv_algo_t 
             ST(build_parts(P, trans, s));
             ST(build_slices(P, trans, lanes, s));
             (trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].kept = true;
-            if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].form == Levels::kLevelOrder)
+            if ((trans ? P->trn : P->fwd).qs[log2_lanes(lanes)].form != Levels::kSliced)
                 ST(build_permuted(P, trans, s));
             break;
         case SPTRSV_ALGO_SELF_COLUMN: ST(build_column(P, trans, s)); break;

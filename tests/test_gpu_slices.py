@@ -155,3 +155,29 @@ def test_a_recorded_update_covers_every_copy_on_every_replay():
                 assert torch.equal(p.solve(b, algo="partitioned"), want), lanes
                 assert torch.equal(p.solve(b, algo="permuted"), want), lanes
             assert torch.equal(x, want)
+
+
+def test_captured_solves_of_a_prepared_width_follow_to_another_array_of_values():
+    """At 32 lanes on rows of two entries (in place unless captured) as at two."""
+    A = synth.lap2d_5pt_lower(400, 410)
+    b = torch.tensor(synth.uniform(A.n, 71), device=dev())
+    with plan_for(A) as p:
+        p.set_partition(4096, 1)
+        graphs = []
+        for lanes in (2, 32):
+            p.set_tuning(lanes, 256, 0)
+            p.prepare("partitioned")
+            x = b.clone()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                p.solve(x, out=x, algo="partitioned")
+            graphs.append((lanes, g, x))
+        first = p.vals
+        p.set_values(2.0 * first)
+        first.fill_(float("nan"))             # nobody reads it any more
+        for lanes, g, x in graphs:
+            p.set_tuning(lanes, 256, 0)
+            x.copy_(b)
+            g.replay()
+            assert torch.equal(x, p.solve(b, algo="self")), lanes
+            assert torch.equal(x, p.solve(b, algo="partitioned")), lanes
