@@ -1150,8 +1150,8 @@ sptrsv_status_t build_parts(sptrsv_plan_t P, bool trans, cudaStream_t s) {
 //    else level-ordered (band of 40, one lane: 28.1 ms, in place 32.5);
 //  * rows are alike and levels wide (more than 512 tickets), so that the empty slots count,
 //    and nearly half of them are empty (7-point 96^3, 16 lanes: 0.97 ms, level-ordered
-//    0.54; but 512 general systems with 8 lanes, whose levels are wide because they are
-//    many: 3.2 ms, level-ordered 7 and more).
+//    0.54; but 200 general systems, 3.1 million rows, 8 lanes, whose levels are wide
+//    because the systems are many: 3.0 ms, level-ordered 8.7).
 // All three give bitwise the same result.
 Levels::Form slice_form(sptrsv_plan_t P, const Levels& L, int lanes, long long slots,
                         const unsigned long long* more) {

@@ -106,8 +106,8 @@ def test_partitioned_solve_of_wide_levels_and_empty_slots():
 
 
 def test_partitioned_solve_of_many_general_systems():
-    """Wide levels because the systems are many: the slices take less than half of what the
-    level-ordered copy takes."""
+    """Wide levels because the systems are many: the slices take a third less than the
+    level-ordered copy (systems of all sizes: two thirds less)."""
     A = synth.block_diagonal([synth.general_lower(4000, 5)] * 200)
     b = torch.tensor(synth.uniform(A.n, 3), device=dev())
     with plan_for(A) as p:
